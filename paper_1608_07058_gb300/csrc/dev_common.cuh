@@ -29,24 +29,118 @@ __device__ __forceinline__ Words4 philox_block(uint32_t k0, uint32_t k1, uint32_
       k0 += 0x9E3779B9u;
       k1 += 0xBB67AE85u;
     }
-    const uint32_t lo_a = 0xD2511F53u * c0;
-    const uint32_t hi_a = __umulhi(0xD2511F53u, c0);
-    const uint32_t lo_b = 0xCD9E8D57u * c2;
-    const uint32_t hi_b = __umulhi(0xCD9E8D57u, c2);
-    const uint32_t n0 = hi_b ^ c1 ^ k0;
-    const uint32_t n2 = hi_a ^ c3 ^ k1;
-    c0 = n0;
-    c1 = lo_b;
-    c2 = n2;
-    c3 = lo_a;
+    // one wide multiplication each (both halves of the product in one instruction)
+    const unsigned long long a = (unsigned long long)0xD2511F53u * c0;
+    const unsigned long long b = (unsigned long long)0xCD9E8D57u * c2;
+    c0 = (uint32_t)(b >> 32) ^ c1 ^ k0;
+    c1 = (uint32_t)b;
+    c2 = (uint32_t)(a >> 32) ^ c3 ^ k1;
+    c3 = (uint32_t)a;
   }
   return Words4{c0, c1, c2, c3};
 }
 
-// FP64 uniform in (0,1) from two words: 52 bits n, u = (n + 1/2) 2^-52 (exact).
+// ---------------------------------------------------------------------------------
+// Exact conversions and comparisons on the integer pipe.  The FP64 unit serves one warp
+// instruction per scheduler in 64 cycles, whatever its active lanes and however many
+// independent ones a warp has, and every conversion to or from a 64-bit type runs on it
+// too (int64 -> float: 64 cycles, 100 of latency; int32 -> float: 4 and 15).  The same
+// values by integer operations take 3 to 12 issue slots.  Results are those of the
+// conversion instructions (round to nearest even); what is out of a fast form's range takes
+// the instruction, as volatile assembly so that it is not executed speculatively.
+// ---------------------------------------------------------------------------------
+
+// float(v), v >= 0: below 2^32 by the 32-bit conversion; above, the top 32 bits with the
+// rest folded into the last one (sticky) round the same way, and the scaling is exact.
+__device__ __forceinline__ float f32_of_count(long long v) {
+  const uint32_t hi = (uint32_t)((unsigned long long)v >> 32), lo = (uint32_t)v;
+  if (hi == 0u) return (float)lo;
+  const int s = __clz((int)hi);  // >= 1: v >= 0
+  const uint32_t top = __funnelshift_l(lo, hi, s) | ((lo << s) != 0u ? 1u : 0u);
+  return (float)top * __int_as_float((159 - s) << 23);
+}
+
+// double(v), v >= 0: below 2^53 by shifting the leading one to bit 52.
+__device__ __forceinline__ double f64_of_count(long long v) {
+  const uint32_t hi = (uint32_t)((unsigned long long)v >> 32), lo = (uint32_t)v;
+  if (hi != 0u) {
+    if (hi < 0x00200000u) {
+      const int s = __clz((int)hi) - 11;
+      return __longlong_as_double((v << s) + ((long long)(1074 - s) << 52));
+    }
+    double d;
+    asm volatile("cvt.rn.f64.s64 %0, %1;" : "=d"(d) : "l"(v));
+    return d;
+  }
+  const int s = __clz((int)lo);
+  const uint32_t m = lo << (s & 31);
+  const uint32_t h = lo ? (m >> 11) + ((uint32_t)(1053 - s) << 20) : 0u;
+  return __hiloint2double((int)h, (int)(lo ? m << 21 : 0u));
+}
+
+// double(f): normal numbers and zero.
+__device__ __forceinline__ double f64_of_f32(float f) {
+  const uint32_t u = __float_as_uint(f), a = u & 0x7fffffffu;
+  if (a - 0x00800000u < 0x7f000000u)
+    return __hiloint2double((int)((u & 0x80000000u) | ((a >> 3) + 0x38000000u)), (int)(u << 29));
+  if (a == 0u) return __hiloint2double((int)u, 0);
+  double d;
+  asm volatile("cvt.f64.f32 %0, %1;" : "=d"(d) : "f"(f));
+  return d;
+}
+
+// float(d), round to nearest even: results in the normal range and zero.
+__device__ __forceinline__ float f32_of_f64(double d) {
+  const uint32_t hi = (uint32_t)__double2hiint(d), lo = (uint32_t)__double2loint(d);
+  const uint32_t a = hi & 0x7fffffffu;
+  if (a - 0x38100000u < 0x0fd00000u) {  // exponents -126 .. 126: rounding cannot overflow
+    const uint32_t m = ((a - 0x38000000u) << 3) | (lo >> 29), rest = lo & 0x1fffffffu;
+    const uint32_t up = (rest + (m & 1u)) > 0x10000000u ? 1u : 0u;
+    return __uint_as_float((hi & 0x80000000u) | (m + up));
+  }
+  if ((a | lo) == 0u) return __uint_as_float(hi);
+  float f;
+  asm volatile("cvt.rn.f32.f64 %0, %1;" : "=f"(f) : "d"(d));
+  return f;
+}
+
+// double(k), 32-bit, exact.
+__device__ __forceinline__ double f64_of_i32(int k) {
+  const uint32_t a = (uint32_t)(k < 0 ? -k : k);
+  const int s = __clz((int)a);
+  const uint32_t m = a << (s & 31);
+  const uint32_t h = ((uint32_t)k & 0x80000000u) | ((m >> 11) + ((uint32_t)(1053 - s) << 20));
+  return __hiloint2double((int)(a ? h : 0u), (int)(m << 21));
+}
+
+// a < b for a >= 0 (not -0) and b not NaN: as integers.
+__device__ __forceinline__ bool f64_lt_nn(double a, double b) {
+  return __double_as_longlong(a) < __double_as_longlong(b);
+}
+
+// a < b for operands that are each in [0, +inf] (not -0) or NaN.
+__device__ __forceinline__ bool f64_lt_pos(double a, double b) {
+  const unsigned long long m = 0x7fffffffffffffffULL, inf = 0x7ff0000000000000ULL;
+  const unsigned long long ub = (unsigned long long)__double_as_longlong(b) & m;
+  return ((unsigned long long)__double_as_longlong(a) & m) < ub && ub <= inf;
+}
+
+// abs(a) > abs(b) (false when a is NaN; b is not NaN).
+__device__ __forceinline__ bool f64_abs_gt(double a, double b) {
+  const unsigned long long m = 0x7fffffffffffffffULL, inf = 0x7ff0000000000000ULL;
+  const unsigned long long ua = (unsigned long long)__double_as_longlong(a) & m;
+  const unsigned long long ub = (unsigned long long)__double_as_longlong(b) & m;
+  return ua > ub && ua <= inf;
+}
+
+// FP64 uniform in (0,1) from two words: 52 bits n, u = (n + 1/2) 2^-52 (exact): the odd
+// integer 2n + 1 shifted so that its leading one is the implicit bit.
 __device__ __forceinline__ double u01_f64(uint32_t hi, uint32_t lo) {
-  const double n = (double)(hi >> 6) * 67108864.0 + (double)(lo >> 6);
-  return (n + 0.5) * 0x1p-52;
+  const unsigned long long v =
+      ((((unsigned long long)(hi >> 6) << 26) | (unsigned long long)(lo >> 6)) << 1) | 1ULL;
+  const int s = __clzll((long long)v);  // >= 11
+  return __longlong_as_double(
+      (long long)((v << (s - 11)) + ((unsigned long long)(1032 - s) << 52)));
 }
 
 // FP32 uniform in (0,1) from one word: 23 bits n, u = (n + 1/2) 2^-23 (exact).
@@ -64,15 +158,27 @@ namespace refmath {
 constexpr double kLn2Head = 0x1.62e42fee00000p-1;   // 32 leading bits of ln 2
 constexpr double kLn2Tail = 0x1.a39ef35793c76p-33;  // ln 2 - kLn2Head
 constexpr double kInvLn2 = 0x1.71547652b82fep+0;
-constexpr double kSqrt2 = 0x1.6a09e667f3bcdp+0;
+constexpr unsigned long long kSqrt2Frac = 0x6a09e667f3bcdULL;  // fraction bits of sqrt 2
 constexpr double kHalfLog2Pi = 0x1.d67f1c864beb5p-1;
 
 // exp(x) on [-708, 709]: x = k ln2 + r, Taylor series of e^r to r^13 by Horner.
 __device__ __forceinline__ double exp_ref(double x) {
-  if (x != x) return x;
-  if (x < -708.0) return 0.0;
-  if (x > 709.0) return __longlong_as_double(0x7ff0000000000000LL);
-  const double kd = floor(x * kInvLn2 + 0.5);
+  // the range by the high word: |x| below 708 needs no further test
+  if ((uint32_t)(__double2hiint(x) & 0x7fffffff) >= 0x40862000u) {
+    if (x != x) return x;
+    if (x < -708.0) return 0.0;
+    if (x > 709.0) return __longlong_as_double(0x7ff0000000000000LL);
+  }
+  const double kx = x * kInvLn2 + 0.5;
+  // floor and its integer, by integer operations (|kx| < 1024)
+  const uint32_t kh = (uint32_t)__double2hiint(kx), kl = (uint32_t)__double2loint(kx);
+  const int ke = (int)((kh >> 20) & 0x7ffu) - 1023;
+  const uint32_t km = (kh & 0xfffffu) | 0x100000u;
+  int k = ke < 0 ? 0 : (int)(km >> (20 - ke));
+  const bool frac = ke < 0 ? ((kh & 0x7fffffffu) | kl) != 0u
+                           : ((km & ((1u << (20 - ke)) - 1u)) | kl) != 0u;
+  if (kh >> 31) k = -k - (frac ? 1 : 0);
+  const double kd = f64_of_i32(k);
   const double r = (x - kd * kLn2Head) - kd * kLn2Tail;
   double p = 1.0 / 6227020800.0;
   p = p * r + 1.0 / 479001600.0;
@@ -88,24 +194,24 @@ __device__ __forceinline__ double exp_ref(double x) {
   p = p * r + 0.5;
   p = p * r + 1.0;
   p = p * r + 1.0;
-  const long long k = (long long)kd;
-  return p * __longlong_as_double((k + 1023LL) << 52);
+  return p * __hiloint2double((k + 1023) << 20, 0);
 }
 
 // log(x) for positive normal x: x = 2^e m, m in [sqrt(1/2), sqrt(2)); with f = m - 1 and
 // s = f/(2+f), log m = 2 atanh s = 2s (1 + z/3 + ... + z^11/23), z = s^2.
 __device__ __forceinline__ double log_ref(double x) {
-  if (x != x || x < 0.0) return __longlong_as_double(0x7ff8000000000000LL);
-  if (x == 0.0) return __longlong_as_double((long long)0xfff0000000000000ULL);
-  if (x == __longlong_as_double(0x7ff0000000000000LL)) return x;
-  const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
-  int e = (int)((bits >> 52) & 0x7ffULL) - 1023;
-  double m = __longlong_as_double(
-      (long long)((bits & 0x000fffffffffffffULL) | 0x3ff0000000000000ULL));
-  if (m > kSqrt2) {
-    m = m * 0.5;
-    e = e + 1;
+  const long long sb = __double_as_longlong(x);
+  if (sb <= 0LL || sb >= 0x7ff0000000000000LL) {  // zero, negative, infinity, NaN
+    if (x != x || x < 0.0) return __longlong_as_double(0x7ff8000000000000LL);
+    if (x == 0.0) return __longlong_as_double((long long)0xfff0000000000000ULL);
+    return x;
   }
+  // mantissa in [1, 2) above sqrt 2 is halved: the comparison and the halving on its bits
+  const unsigned long long bits = (unsigned long long)sb, frac = bits & 0x000fffffffffffffULL;
+  const bool above = frac > kSqrt2Frac;
+  const int e = (int)(bits >> 52) - (above ? 1022 : 1023);
+  const double m = __longlong_as_double(
+      (long long)(frac | (above ? 0x3fe0000000000000ULL : 0x3ff0000000000000ULL)));
   const double f = m - 1.0;
   const double s = f / (2.0 + f);
   const double z = s * s;
@@ -122,7 +228,7 @@ __device__ __forceinline__ double log_ref(double x) {
   q = q * z + 1.0 / 3.0;
   const double two_s = s + s;
   const double logm = two_s + (two_s * z) * q;
-  const double ed = (double)e;
+  const double ed = f64_of_i32(e);
   return ed * kLn2Head + (ed * kLn2Tail + logm);
 }
 

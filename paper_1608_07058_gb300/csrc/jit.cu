@@ -18,6 +18,7 @@
 #include <vector>
 
 #include "jit.h"
+#include "ml_internal.h"
 #include "jit_sources.h"  // generated by the build: the kernel headers as strings
 
 namespace mlk {
@@ -58,6 +59,31 @@ std::string table1(const char* name, const char* type, int n, F value) {
 
 }  // namespace
 
+namespace {
+// The reaction holding each reaction's integral G: the lowest one with the same reactants
+// (entries beyond M: reaction 0, which is never their own).
+std::vector<int> g_owners(int N, int M, int MM, const int32_t* ord) {
+  std::vector<int> own(MM, 0);
+  for (int j = 0; j < M; ++j) {
+    own[j] = j;
+    for (int i = 0; i < j && own[j] == j; ++i)
+      if (std::memcmp(ord + i * N, ord + j * N, sizeof(int32_t) * N) == 0) own[j] = i;
+  }
+  return own;
+}
+
+int g_owner_count(const std::vector<int>& own, int M) {
+  int n = 0;
+  for (int j = 0; j < M; ++j) n += own[j] == j;
+  return n;
+}
+}  // namespace
+
+int jit_pool_words(const JitSpec& k) {
+  const int n = g_owner_count(g_owners(k.N, k.M, k.MM, k.ord), k.M);
+  return lane_record_words(k.NM, k.MM, k.precision_ref) - 2 * (k.MM - n);
+}
+
 std::string jit_source(const JitSpec& k) {
   const int NM = k.NM, MM = k.MM;
   auto in = [&](int j, int s) { return j < k.M && s < k.N; };
@@ -90,6 +116,9 @@ std::string jit_source(const JitSpec& k) {
   src += table1("hor", "uint8_t", NM, [&](int s) {
     return std::to_string(s < k.N ? (int)k.hor[s] : 0);
   });
+  const std::vector<int> gown = g_owners(k.N, k.M, MM, k.ord);
+  src += "  static constexpr int n_gown = " + std::to_string(g_owner_count(gown, k.M)) + ";\n";
+  src += table1("gown", "int8_t", MM, [&](int j) { return std::to_string(gown[j]); });
   src += table1("rates", "double", MM, [&](int j) {
     return j < k.M ? hexd(k.rates[j]) : std::string("0.0");
   });

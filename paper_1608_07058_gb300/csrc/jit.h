@@ -27,6 +27,10 @@ struct JitSpec {
   bool occ = false;
 };
 
+// 32-bit words of a trajectory's record in the specialized pool kernel: without the
+// integrals of reactions that share another one's reactants.
+int jit_pool_words(const JitSpec& k);
+
 // CUDA source of the kernel `ml_jit_kernel(const void* tables, SimArgs)` for spec k.
 std::string jit_source(const JitSpec& k);
 

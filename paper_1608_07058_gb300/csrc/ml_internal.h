@@ -54,6 +54,9 @@ struct alignas(16) ThreadModel {
   static constexpr bool kCompiled = false;  // tables read at run time (see JitModel)
   double rates[MM];
   float nuf[MM][NM];    // nu_js as FP32 (updates of the fast SSA slice's FP32 state copy)
+  // reactants of reaction j in one word, in increasing species: byte k = species of the
+  // k-th (low nibble) and its multiplicity (high nibble), byte 3 = their number (0..3)
+  uint32_t rx[MM];
   int8_t ord[MM][NM];   // m_js
   int8_t nu[MM][NM];    // nu_js
   int8_t partner[MM];   // for the lower reaction of a reversible pair: the other; else -1
@@ -137,6 +140,12 @@ struct SimArgs {
   const double* t_obs;
   int64_t* X_obs;
   int32_t K_obs;
+  // trajectories a warp runs at a time (thread kernels): 1..32 lanes of the round-based and
+  // sequential drivers, 1..kPoolSlots records of the pool driver
+  int32_t per_warp;
+  // the control parameters that fast precision compares in FP32, rounded once on the host
+  // (a double -> float conversion runs on the FP64 unit)
+  float eps_f, ssa_factor_f, pe_delta_f, stiff_ratio_f;
 };
 
 #ifndef __CUDACC_RTC__

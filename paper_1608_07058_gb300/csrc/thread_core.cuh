@@ -31,21 +31,22 @@ namespace mlk {
 template <int MM, class R>
 __device__ __forceinline__ R lane_tree_sum(const R (&v)[MM]) {
   static_assert(MM <= 32, "thread variant holds at most 32 reactions");
-  R lane[32];
+  // the additions of empty lanes' zeros are left out (the elements are not negative, so
+  // v + 0 is v): MM - 1 additions instead of 31
+  R lane[MM];
 #pragma unroll
-  for (int l = 0; l < 32; ++l) lane[l] = (l < MM) ? v[l] : R(0);
+  for (int l = 0; l < MM; ++l) lane[l] = v[l];
 #pragma unroll
   for (int d = 16; d >= 1; d >>= 1) {
 #pragma unroll
-    for (int l = 0; l < d; ++l) lane[l] = lane[l] + lane[l + d];
+    for (int l = 0; l < d; ++l)
+      if (l + d < MM) lane[l] = lane[l] + lane[l + d];
   }
   return lane[0];
 }
 
 // Sum over reactions: the canonical lane tree in reference precision (bitwise parity with
-// the CPU reference); fast precision may add in any order and adds sequentially (the tree
-// over 32 lanes costs 31 additions, most of them of zeros that IEEE arithmetic cannot
-// drop).
+// the CPU reference); fast precision may add in any order and adds sequentially.
 template <int MM, class R, bool kRef>
 __device__ __forceinline__ R reaction_sum(const R (&v)[MM]) {
   if (kRef) return lane_tree_sum<MM, R>(v);
@@ -55,12 +56,29 @@ __device__ __forceinline__ R reaction_sum(const R (&v)[MM]) {
   return s;
 }
 
+// A count as the working precision (x >= 0), without the FP64 unit.
+template <class R>
+__device__ __forceinline__ R of_count(long long x);
+template <>
+__device__ __forceinline__ float of_count<float>(long long x) { return f32_of_count(x); }
+template <>
+__device__ __forceinline__ double of_count<double>(long long x) { return f64_of_count(x); }
+
 // C(v, m) for m = 1, 2, 3 on a real argument, in this operation order.
 template <class R>
 __device__ __forceinline__ R comb_factor(R v, int m) {
   if (m == 1) return v;
   if (m == 2) return (v * (v - R(1))) * R(0.5);
   return ((v * (v - R(1))) * (v - R(2))) / R(6);
+}
+
+// C(x, m) of a count: as comb_factor on the converted count.  In FP64 C(x, 2) is an integer
+// operation while x (x - 1) stays below 2^53, where every step of comb_factor is exact.
+template <class R>
+__device__ __forceinline__ R comb_count(long long x, int m) {
+  if (sizeof(R) == 8 && m == 2 && x < 94906265LL)
+    return of_count<R>((long long)(((unsigned long long)x * (unsigned long long)(x - 1)) >> 1));
+  return comb_factor<R>(of_count<R>(x), m);
 }
 
 // d/dv C(v, m): 1, v - 1/2, (3 v^2 - 6 v + 2) / 6, in this operation order.
@@ -125,25 +143,29 @@ __device__ __forceinline__ void kahan_add(float& s, float& c, float v) {
   s = t;
 }
 
+// a < b for values in [0, +inf] (not -0) or NaN
+__device__ __forceinline__ bool lt_pos(double a, double b) { return f64_lt_pos(a, b); }
+__device__ __forceinline__ bool lt_pos(float a, float b) { return a < b; }
+
 // Highest-order-reaction factor h_s (Cao 2006) from the species' flags and count.
 template <class R>
 __device__ __forceinline__ R hor_factor(uint8_t f, long long x) {
-  const R xd = (R)x;
+  const R xd = of_count<R>(x);
   R h = R(0);
-  if (f & kHorO1) h = h < R(1) ? R(1) : h;
-  if (f & kHorO2M1) h = h < R(2) ? R(2) : h;
+  if (f & kHorO1) h = lt_pos(h, R(1)) ? R(1) : h;
+  if (f & kHorO2M1) h = lt_pos(h, R(2)) ? R(2) : h;
   if (f & kHorO2M2) {
     const R v = x >= 2 ? R(2) + R(1) / (xd - R(1)) : R(2);
-    h = h < v ? v : h;
+    h = lt_pos(h, v) ? v : h;
   }
-  if (f & kHorO3M1) h = h < R(3) ? R(3) : h;
+  if (f & kHorO3M1) h = lt_pos(h, R(3)) ? R(3) : h;
   if (f & kHorO3M2) {
     const R v = x >= 2 ? R(1.5) * (R(2) + R(1) / (xd - R(1))) : R(3);
-    h = h < v ? v : h;
+    h = lt_pos(h, v) ? v : h;
   }
   if (f & kHorO3M3) {
     const R v = x >= 3 ? (R(3) + R(1) / (xd - R(1))) + R(2) / (xd - R(2)) : R(3);
-    h = h < v ? v : h;
+    h = lt_pos(h, v) ? v : h;
   }
   return h;
 }
@@ -151,9 +173,27 @@ __device__ __forceinline__ R hor_factor(uint8_t f, long long x) {
 struct PrecRef {
   using R = double;
   static constexpr bool kRef = true;
+  // a b rounded, and a b + c with the product rounded, whatever the compiler would contract
+  __device__ static __forceinline__ R mul(R a, R b) { return __dmul_rn(a, b); }
+  __device__ static __forceinline__ R mad(R a, R b, R c) { return __dadd_rn(__dmul_rn(a, b), c); }
   __device__ static __forceinline__ R u(const Words4& w, int k) {
     return k == 0 ? u01_f64(w.w0, w.w1) : u01_f64(w.w2, w.w3);
   }
+  // comparisons of values in [0, +inf] (not -0) or NaN, on the integer pipe
+  __device__ static __forceinline__ bool lt(R a, R b) { return f64_lt_pos(a, b); }
+  __device__ static __forceinline__ bool positive(R a) { return f64_lt_pos(0.0, a); }
+  __device__ static __forceinline__ bool zero(R a) {
+    return (__double_as_longlong(a) << 1) == 0;
+  }
+  __device__ static __forceinline__ bool negative(R a) {  // below zero (-0 is not)
+    return __double_as_longlong(a) < 0 && !zero(a);
+  }
+  __device__ static __forceinline__ R of_f64(double v) { return v; }
+  __device__ static __forceinline__ double to_f64(R v) { return v; }
+  __device__ static __forceinline__ R eps(const SimArgs& A) { return A.eps; }
+  __device__ static __forceinline__ R ssa_factor(const SimArgs& A) { return A.ssa_factor; }
+  __device__ static __forceinline__ R pe_delta(const SimArgs& A) { return A.pe_delta; }
+  __device__ static __forceinline__ R stiff_ratio(const SimArgs& A) { return A.stiff_ratio; }
   __device__ static __forceinline__ R log(R x) { return refmath::log_ref(x); }
   __device__ static __forceinline__ R exp(R x) { return refmath::exp_ref(x); }
   __device__ static __forceinline__ R lfact(long long k) {
@@ -169,9 +209,22 @@ struct PrecRef {
 struct PrecFast {
   using R = float;
   static constexpr bool kRef = false;
+  // a b rounded, and a b + c fused, whatever the compiler would contract
+  __device__ static __forceinline__ R mul(R a, R b) { return __fmul_rn(a, b); }
+  __device__ static __forceinline__ R mad(R a, R b, R c) { return __fmaf_rn(a, b, c); }
   __device__ static __forceinline__ R u(const Words4& w, int k) {
     return k == 0 ? u01_f32(w.w0) : u01_f32(w.w2);
   }
+  __device__ static __forceinline__ bool lt(R a, R b) { return a < b; }
+  __device__ static __forceinline__ bool positive(R a) { return a > 0.f; }
+  __device__ static __forceinline__ bool zero(R a) { return a == 0.f; }
+  __device__ static __forceinline__ bool negative(R a) { return a < 0.f; }
+  __device__ static __forceinline__ R of_f64(double v) { return f32_of_f64(v); }
+  __device__ static __forceinline__ double to_f64(R v) { return f64_of_f32(v); }
+  __device__ static __forceinline__ R eps(const SimArgs& A) { return A.eps_f; }
+  __device__ static __forceinline__ R ssa_factor(const SimArgs& A) { return A.ssa_factor_f; }
+  __device__ static __forceinline__ R pe_delta(const SimArgs& A) { return A.pe_delta_f; }
+  __device__ static __forceinline__ R stiff_ratio(const SimArgs& A) { return A.stiff_ratio_f; }
   // accurate logf: the waiting times -log(u)/a0 need relative accuracy for u near 1,
   // where the hardware approximation's absolute error would bias the clock
   __device__ static __forceinline__ R log(R x) { return logf(x); }
@@ -189,6 +242,10 @@ struct PrecFast {
 struct PrecWide {
   using R = double;
   static constexpr bool kRef = false;
+  // a b rounded, and a b + c fused, whatever the compiler would contract
+  __device__ static __forceinline__ R mul(R a, R b) { return __dmul_rn(a, b); }
+  __device__ static __forceinline__ R mad(R a, R b, R c) { return __fma_rn(a, b, c); }
+  __device__ static __forceinline__ bool negative(R a) { return PrecRef::negative(a); }
   __device__ static __forceinline__ R u(const Words4& w, int k) {
     return k == 0 ? u01_f64(w.w0, w.w1) : u01_f64(w.w2, w.w3);
   }
@@ -204,69 +261,277 @@ struct PrecWide {
 
 constexpr int kPtrsMaxTrials = 256;
 
-// PTRS: Hoermann (1993), transformed rejection with squeeze, for mean mu >= 10.  Trial b
-// uses block b of the stream: U from the first uniform, V from the second.
 struct PoissonDraw {
   long long k;
   uint32_t flags;  // ML_ST_PTRS_CAP when the trial cap was hit
 };
 
+// The integer of a non-negative integral value.
+__device__ __forceinline__ long long count_of(float v) {
+  if (v < 2147483648.f) return (long long)(int)v;
+  long long k;
+  asm volatile("cvt.rzi.s64.f32 %0, %1;" : "=l"(k) : "f"(v));
+  return k;
+}
+__device__ __forceinline__ long long count_of(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  const int e = (int)(b >> 52) - 1023;  // sign 0
+  if (e < 0) return 0;
+  const unsigned long long m = (b & 0x000fffffffffffffULL) | 0x0010000000000000ULL;
+  if (e <= 52) return (long long)(m >> (52 - e));
+  long long k;
+  asm volatile("cvt.rzi.s64.f64 %0, %1;" : "=l"(k) : "d"(v));
+  return k;
+}
+
+// PTRS: Hoermann (1993), transformed rejection with squeeze, for mean mu >= 10.  Trial b
+// uses block b of the stream: U from the first uniform, V from the second.
+
+// The acceptance test beyond the squeeze, in the precision's own arithmetic.
+template <class P>
+__device__ __noinline__ bool ptrs_accept(typename P::R mu, typename P::R a, typename P::R b,
+                                         typename P::R us, typename P::R V, typename P::R kd) {
+  using R = typename P::R;
+  const R inv_alpha = R(1.1239) + R(1.1328) / (b - R(3.4));
+  const R lhs = (P::log(V) + P::log(inv_alpha)) - P::log(a / (us * us) + b);
+  R rhs;
+  if (P::kRef || lt_pos(kd, R(10))) {
+    const R loglam = P::log(mu);
+    rhs = (-mu + kd * loglam) - P::lfact(count_of(kd));
+  } else {
+    // log of the Poisson pmf without cancellation: with z = k + 1 and Stirling's series
+    // for log Gamma(z), -mu + k log mu - log k! =
+    //   (z - mu) + (z - 1) log1p((mu - z)/z) - log(z)/2 - log(2 pi)/2 - 1/(12 z) + 1/(360 z^3)
+    const R z = kd + R(1);
+    const R iz = R(1) / z;
+    rhs = ((z - mu) + (z - R(1)) * P::log1p((mu - z) * iz)) - R(0.5) * P::log(z) -
+          R(0.91893853320467274178) - iz * (R(1) / R(12) - (iz * iz) * (R(1) / R(360)));
+  }
+  return lhs <= rhs;
+}
+
+// The same test estimated in FP32: 1 accept, -1 reject, 0 too close to tell (then the caller
+// evaluates it in its own arithmetic, so the outcome is that of ptrs_accept).  The four
+// logarithms of the exact test cost about 250 instructions on the FP64 unit (16,000 cycles
+// of it) or 150 in FP32; some lane of a warp nearly always needs the test.
+//   lhs = log(V inv_alpha us^2 / (a + b us^2)) by one hardware logarithm;
+//   rhs = z (L - x) - L - log(z)/2 - log(2 pi)/2 - 1/(12 z) + 1/(360 z^3), x = d/z, d = mu - z,
+//   L = log1p(x): since z - mu = -z x, the large terms cancel before they are formed, and for
+//   |x| < 1/4 L - x is its series to x^8 (relative error below 2e-5).
+// Errors: Stirling's series 8e-4 at z = 1; the estimate 1e-4 of |z (L - x)| with room; the
+// FP32 form of ptrs_accept, which does form z - mu, up to 4e-7 |d|.  us >= 1e-4 here.
+__device__ __forceinline__ int ptrs_estimate(float inv_alpha, float a, float b, float us,
+                                             float V, float z, float d) {
+  const float u2 = us * us;
+  const float lhs = 0.69314718f * __log2f(__fdividef(V * inv_alpha * u2, a + b * u2));
+  const float iz = __fdividef(1.f, z), x = d * iz;
+  float L, t;
+  if (fabsf(x) < 0.25f) {
+    float q = -0.125f;
+    q = q * x + (1.f / 7.f);
+    q = q * x - (1.f / 6.f);
+    q = q * x + 0.2f;
+    q = q * x - 0.25f;
+    q = q * x + (1.f / 3.f);
+    q = q * x - 0.5f;
+    const float s = q * x * x;
+    L = x + s;
+    t = z * s;
+  } else {
+    L = 0.69314718f * __log2f(1.f + x);
+    t = z * (L - x);
+  }
+  const float rhs = t - L - 0.34657359f * __log2f(z) - 0.91893853f -
+                    iz * (0.083333333f - iz * iz * 0.0027777778f);
+  const float gap = rhs - lhs;
+  const float margin = 4.0e-3f + 1.0e-4f * fabsf(t) + 2.0e-6f * fabsf(d);
+  return gap > margin ? 1 : gap < -margin ? -1 : 0;
+}
+
+// One trial in the precision's own arithmetic (FP32: the estimate before the exact test).
+template <class P>
+__device__ __forceinline__ bool ptrs_trial_own(typename P::R mu, const Words4& w, long long& k) {
+  using R = typename P::R;
+  const R slam = P::sqrt(mu);
+  const R b = P::mad(R(2.53), slam, R(0.931));
+  const R a = P::mad(R(0.02483), b, R(-0.059));
+  const R v_r = R(0.9277) - R(3.6224) / (b - R(2));
+  const R U = P::u(w, 0) - R(0.5);
+  const R V = P::u(w, 1);
+  const R us = R(0.5) - fabs(U);  // positive: |U| < 1/2
+  const R kd = floor(P::mad((R(2) * a) / us + b, U, mu) + R(0.43));
+  bool ok = false;
+  if (!lt_pos(us, R(0.07)) && !lt_pos(v_r, V)) {
+    ok = true;
+  } else if (!(P::negative(kd) || (lt_pos(us, R(0.013)) && lt_pos(us, V)))) {
+    int est = 0;
+    if constexpr (sizeof(R) == 4) {
+      const float z = kd + 1.f;
+      if (us > 1.0e-4f)
+        est = ptrs_estimate(1.1239f + __fdividef(1.1328f, b - 3.4f), a, b, us, V, z, mu - z);
+    }
+    ok = est != 0 ? est > 0 : ptrs_accept<P>(mu, a, b, us, V, kd);
+  }
+  if (ok) k = count_of(kd);
+  return ok;
+}
+template <class P>
+__device__ __noinline__ bool ptrs_trial_exact(typename P::R mu, const Words4& w, long long& k) {
+  return ptrs_trial_own<P>(mu, w, k);
+}
+
+// Reference precision: the trial with FP32 setup and FP32 estimates, the proposal
+// k = floor(x) kept to FP64 by adding its FP32 part (relative error below 3e-6) to mu + 0.43;
+// where a floor, a comparison or the test could go either way, the exact trial decides
+// (about 1e-2 of the trials at mu = 1e4).  Four FP64 additions instead of about 60 operations
+// with a square root and three divisions, and 250 more with the test.
+__device__ __forceinline__ bool ptrs_trial_near(double mu, const Words4& w, long long& k) {
+  const long long n1 = ((long long)(w.w0 >> 6) << 26) | (long long)(w.w1 >> 6);
+  const long long n2 = ((long long)(w.w2 >> 6) << 26) | (long long)(w.w3 >> 6);
+  // U = m 2^-53, us = (2^52 - |m|) 2^-53, exact integers
+  const long long m = 2 * n1 + 1 - (1LL << 52);
+  const long long am = m < 0 ? -m : m;
+  const float Ua = f32_of_count(am) * 0x1p-53f, us = f32_of_count((1LL << 52) - am) * 0x1p-53f;
+  const float V = f32_of_count(2 * n2 + 1) * 0x1p-53f;
+  const float b = 0.931f + 2.53f * sqrtf(f32_of_f64(mu));
+  const float a = -0.059f + 0.02483f * b;
+  const float prod = (__fdividef(2.f * a, us) + b) * (m < 0 ? -Ua : Ua);
+  const double kx = (mu + 0.43) + f64_of_f32(prod);
+  const float err = 1.0e-6f + 3.0e-6f * fabsf(prod);
+  if (us > 1.0e-4f && f64_lt_pos(mu, 1.0e9)) {
+    if (__double2hiint(kx) < 0) {  // k < 0: rejected (us < 0.07 there)
+      if (f32_of_f64(-kx) > 1.f + err) return false;
+    } else {
+      k = count_of(kx);
+      const float frac = f32_of_f64(kx - f64_of_count(k));
+      const float v_r = 0.9277f - __fdividef(3.6224f, b - 2.f);
+      if (frac > err && frac < 1.f - err && fabsf(us - 0.07f) > 1.0e-6f &&
+          fabsf(us - 0.013f) > 1.0e-6f) {
+        if (us > 0.07f && V < v_r - 4.0e-6f) return true;
+        if (us < 0.07f || V > v_r + 4.0e-6f) {
+          if (us < 0.013f && V > us + 1.0e-6f) return false;
+          if (us > 0.013f || V < us - 1.0e-6f) {
+            const double z = f64_of_count(k + 1);
+            const int est =
+                ptrs_estimate(1.1239f + __fdividef(1.1328f, b - 3.4f), a, b, us, V,
+                              f32_of_count(k + 1), f32_of_f64(mu - z));
+            if (est != 0) return est > 0;
+          }
+        }
+      }
+    }
+  }
+  return ptrs_trial_exact<PrecRef>(mu, w, k);
+}
+
+template <class P>
+__device__ __forceinline__ bool ptrs_trial(typename P::R mu, const Words4& w, long long& k) {
+  if constexpr (P::kRef) return ptrs_trial_near(mu, w, k);
+  else return ptrs_trial_own<P>(mu, w, k);
+}
+
 template <class P>
 __device__ __noinline__ PoissonDraw poisson_ptrs(typename P::R mu, uint32_t k0, uint32_t k1,
                                                  uint32_t id, uint32_t step, uint32_t stream) {
   using R = typename P::R;
-  const R slam = P::sqrt(mu);
-  const R loglam = P::log(mu);
-  const R b = R(0.931) + R(2.53) * slam;
-  const R a = R(-0.059) + R(0.02483) * b;
-  const R inv_alpha = R(1.1239) + R(1.1328) / (b - R(3.4));
-  const R v_r = R(0.9277) - R(3.6224) / (b - R(2));
-  for (uint32_t trial = 0; trial < (uint32_t)kPtrsMaxTrials; ++trial) {
-    const Words4 w = philox_block(k0, k1, id, step, stream, trial);
-    const R U = P::u(w, 0) - R(0.5);
-    const R V = P::u(w, 1);
-    const R us = R(0.5) - fabs(U);
-    const R kd = floor((((R(2) * a) / us + b) * U + mu) + R(0.43));
-    if (us >= R(0.07) && V <= v_r) return PoissonDraw{(long long)kd, 0u};
-    if (kd < R(0) || (us < R(0.013) && V > us)) continue;
-    const R lhs = (P::log(V) + P::log(inv_alpha)) - P::log(a / (us * us) + b);
-    R rhs;
-    if (P::kRef || kd < R(10)) {
-      rhs = (-mu + kd * loglam) - P::lfact((long long)kd);
-    } else {
-      // log of the Poisson pmf without cancellation: with z = k + 1 and Stirling's series
-      // for log Gamma(z), -mu + k log mu - log k! =
-      //   (z - mu) + (z - 1) log1p((mu - z)/z) - log(z)/2 - log(2 pi)/2 - 1/(12 z) + 1/(360 z^3)
-      const R z = kd + R(1);
-      const R iz = R(1) / z;
-      rhs = ((z - mu) + (z - R(1)) * P::log1p((mu - z) * iz)) - R(0.5) * P::log(z) -
-            R(0.91893853320467274178) - iz * (R(1) / R(12) - (iz * iz) * (R(1) / R(360)));
-    }
-    if (lhs <= rhs) return PoissonDraw{(long long)kd, 0u};
-  }
+  long long k = 0;
+  for (uint32_t trial = 0; trial < (uint32_t)kPtrsMaxTrials; ++trial)
+    if (ptrs_trial<P>(mu, philox_block(k0, k1, id, step, stream, trial), k))
+      return PoissonDraw{k, 0u};
   return PoissonDraw{(long long)floor(mu + R(0.5)), ML_ST_PTRS_CAP};
 }
 
-// Poisson(mu): 0 for mu <= 0 (no draw); inversion by sequential search below 10; PTRS.
+// mu / k rounded to nearest, for mu in (2^-60, 10) and an integer k >= 1: with z near 1/k
+// (relative error below 2^-20 in FP32, 2^-50 in FP64), q = mu z and the remainder
+// r = mu - k q (exact: one FMA), q + r z misses mu / k by far less than the smallest
+// distance of mu / k from a midpoint of two numbers: mu / k = c/k ulps with an integer c, so
+// it is no midpoint (k times an odd half-integer of the quotient's precision does not fit
+// the significand of mu) and at least 1/(2k) ulp away from one.  So the result is that
+// of the IEEE division, in 4 instructions instead of about 10 (FP32) and in 3 on the
+// FP64 unit instead of 9 and a conversion of k.
+__device__ __forceinline__ float div_by_int(float mu, int k) {
+  const float kf = (float)k;
+  const float z = __fdividef(1.f, kf);
+  const float q = __fmul_rn(mu, z);
+  return __fmaf_rn(__fmaf_rn(-kf, q, mu), z, q);
+}
+constexpr int kRecips = 48;
+struct Recips {
+  double v[kRecips];
+};
+constexpr Recips make_recips() {
+  Recips t{};
+  t.v[0] = 0.0;
+  for (int k = 1; k < kRecips; ++k) t.v[k] = 1.0 / (double)k;
+  return t;
+}
+__constant__ constexpr Recips kRecip = make_recips();
+__device__ __forceinline__ double div_by_int(double mu, int k) {
+  const double kd = f64_of_i32(k);
+  if (k >= kRecips) return mu / kd;
+  const double z = kRecip.v[k];
+  const double q = __dmul_rn(mu, z);
+  return __fma_rn(__fma_rn(-kd, q, mu), z, q);
+}
+
+// Means below 10: inversion by sequential search (mu > 0).
+template <class P>
+__device__ __forceinline__ int poisson_invert(typename P::R mu, typename P::R u) {
+  using R = typename P::R;
+  R p = P::exp(-mu);
+  R F = p;
+  int k = 0;
+  while (P::lt(F, u)) {
+    k = k + 1;
+    p = p * div_by_int(mu, k);
+    if (P::zero(p)) break;
+    F = F + p;
+  }
+  return k;
+}
+__device__ __noinline__ inline int poisson_invert_exact(double mu, double u) {
+  return poisson_invert<PrecRef>(mu, u);
+}
+// Reference precision: the search in FP32 first.  The FP32 cumulative sums are within 2e-6 of
+// the FP64 ones (an exponential, at most 60 products and sums), so while u stays farther
+// than 1e-5 from each of them the FP64 search makes the same steps; otherwise (a few 1e-4 of
+// the draws) it runs: an exponential of about 30 FP64 operations and five more per step.
+__device__ __forceinline__ int poisson_invert_near(double mu, double u) {
+  const float m = f32_of_f64(mu), uf = f32_of_f64(u);
+  float p = __expf(-m), F = p;
+  int k = 0;
+  bool clear = fabsf(uf - F) > 1.0e-5f;
+  while (F < uf && clear && k < 60) {
+    ++k;
+    p = p * __fdividef(m, (float)k);
+    F = F + p;
+    clear = fabsf(uf - F) > 1.0e-5f;
+  }
+  return clear && k < 60 ? k : poisson_invert_exact(mu, u);
+}
+
+template <class P>
+__device__ __forceinline__ int poisson_invert_at(typename P::R mu, typename P::R u) {
+  if constexpr (P::kRef) return poisson_invert_near(mu, u);
+  else return poisson_invert<P>(mu, u);
+}
+
+// Poisson(mu) for mu < 10: 0 for mu <= 0 (no draw).
+template <class P>
+__device__ __noinline__ int poisson_small(typename P::R mu, uint32_t k0, uint32_t k1,
+                                          uint32_t id, uint32_t step, uint32_t stream) {
+  if (!P::positive(mu)) return 0;
+  const Words4 w = philox_block(k0, k1, id, step, stream, 0);
+  return poisson_invert_at<P>(mu, P::u(w, 0));
+}
+
+// Poisson(mu): inversion by sequential search below 10; PTRS.
 template <class P>
 __device__ __forceinline__ PoissonDraw poisson_sample(typename P::R mu, uint32_t k0, uint32_t k1,
                                                    uint32_t id, uint32_t step, uint32_t stream) {
   using R = typename P::R;
-  if (!(mu > R(0))) return PoissonDraw{0, 0u};
-  if (mu < R(10)) {
-    const Words4 w = philox_block(k0, k1, id, step, stream, 0);
-    const R u = P::u(w, 0);
-    R p = P::exp(-mu);
-    R F = p;
-    long long k = 0;
-    while (u > F) {
-      k = k + 1;
-      p = p * (mu / (R)k);
-      if (p == R(0)) break;
-      F = F + p;
-    }
-    return PoissonDraw{k, 0u};
-  }
+  if (!P::positive(mu) || P::lt(mu, R(10)))
+    return PoissonDraw{(long long)poisson_small<P>(mu, k0, k1, id, step, stream), 0u};
   return (!P::kRef && mu > R(4.0e6)) ? poisson_ptrs<PrecWide>((double)mu, k0, k1, id, step, stream)
                                      : poisson_ptrs<P>(mu, k0, k1, id, step, stream);
 }
@@ -280,6 +545,16 @@ __device__ __forceinline__ long long poisson_draw(typename P::R mu, uint32_t k0,
   return d.k;
 }
 
+// |a| > |b| (false when a is NaN)
+__device__ __forceinline__ bool abs_gt(double a, double b) { return f64_abs_gt(a, b); }
+__device__ __forceinline__ bool abs_gt(float a, float b) { return fabsf(a) > fabsf(b); }
+
+// v t for a net change v: the common changes by one are exact without a product.
+__device__ __forceinline__ double nu_times(int v, double t) {
+  return v == 1 ? t : v == -1 ? -t : f64_of_i32(v) * t;
+}
+__device__ __forceinline__ float nu_times(int v, float t) { return (float)v * t; }
+
 // MDL: the model tables' type -- the shared-memory ThreadModel staged at kernel start, or
 // a type with the same members known at compile time.
 template <int NM, int MM, class P, class MDL = ThreadModel<NM, MM>>
@@ -287,45 +562,94 @@ struct ThreadTraj {
   using R = typename P::R;
   using Model = MDL;
 
-  // g_j at an integer state (0 when some x_s < m_js), product in increasing s.
-  __device__ static __forceinline__ R g_int(const Model& md, int j, const long long (&x)[NM]) {
-    R v = R(1);
+  // g_j of a state by the table's reactant word: comb(x_s, m) of the k-th reactant, the
+  // product in increasing s, 0 when some x_s < m_js.  The code is a tenth of the loop over
+  // all (reaction, species) pairs with a branch per order, which the precompiled kernels
+  // ran before: their stalls were instruction fetch.
+  template <class V, class F>
+  __device__ static __forceinline__ auto g_word(uint32_t rx, const V (&x)[NM], F comb) {
+    using O = decltype(comb(x[0], 1));
+    O v = O(1);
     bool zero = false;
+    const int nr = (int)(rx >> 24);
 #pragma unroll
-    for (int s = 0; s < NM; ++s) {
-      const int m = md.ord[j][s];
-      if (m != 0) {
-        if (x[s] < m) zero = true;
-        else v = v * comb_factor<R>((R)x[s], m);
+    for (int k = 0; k < 3; ++k) {
+      if (k < nr) {
+        const int sp = (int)(rx >> (8 * k)) & 15, m = (int)(rx >> (8 * k + 4)) & 15;
+        V xs = x[0];
+#pragma unroll
+        for (int s = 1; s < NM; ++s) xs = s == sp ? x[s] : xs;
+        zero = zero || xs < (V)m;
+        const O f = comb(xs, m);
+        v = k == 0 ? f : v * f;
       }
     }
-    return zero ? R(0) : v;
+    return zero ? O(0) : v;
+  }
+
+  // g_j at an integer state (0 when some x_s < m_js), product in increasing s.
+  __device__ static __forceinline__ R g_int(const Model& md, int j, const long long (&x)[NM]) {
+    if constexpr (!Model::kCompiled) {
+      return g_word(md.rx[j], x, [](long long xs, int m) { return comb_count<R>(xs, m); });
+    } else {
+      R v = R(1);
+      bool zero = false;
+#pragma unroll
+      for (int s = 0; s < NM; ++s) {
+        const int m = md.ord[j][s];
+        if (m != 0) {
+          if (x[s] < m) zero = true;
+          else v = v * comb_count<R>(x[s], m);
+        }
+      }
+      return zero ? R(0) : v;
+    }
   }
 
   // Fast precision: g_j from an FP32 copy of the state (exact while counts stay below
   // 2^24, where it equals g_int; above, FP32 rounds the count as g_int's conversion does).
   __device__ static __forceinline__ float g_flt(const Model& md, int j, const float (&xf)[NM]) {
-    float v = 1.f;
-    bool zero = false;
+    if constexpr (!Model::kCompiled) {
+      return g_word(md.rx[j], xf, [](float xs, int m) { return comb_factor<float>(xs, m); });
+    } else {
+      float v = 1.f;
+      bool zero = false;
 #pragma unroll
-    for (int s = 0; s < NM; ++s) {
-      const int m = md.ord[j][s];
-      if (m != 0) {
-        if (xf[s] < (float)m) zero = true;
-        else v = v * comb_factor<float>(xf[s], m);
+      for (int s = 0; s < NM; ++s) {
+        const int m = md.ord[j][s];
+        if (m != 0) {
+          if (xf[s] < (float)m) zero = true;
+          else v = v * comb_factor<float>(xf[s], m);
+        }
       }
+      return zero ? 0.f : v;
     }
-    return zero ? 0.f : v;
   }
 
   // g_j at a real state (implicit solve), FP64 always.
   __device__ static __forceinline__ double g_real(const Model& md, int j,
                                                   const double (&y)[NM]) {
     double v = 1.0;
+    if constexpr (!Model::kCompiled) {
+      const uint32_t rx = md.rx[j];
+      const int nr = (int)(rx >> 24);
 #pragma unroll
-    for (int s = 0; s < NM; ++s) {
-      const int m = md.ord[j][s];
-      if (m != 0) v = v * comb_factor<double>(y[s], m);
+      for (int k = 0; k < 3; ++k) {
+        if (k < nr) {
+          const int sp = (int)(rx >> (8 * k)) & 15, m = (int)(rx >> (8 * k + 4)) & 15;
+          double ys = y[0];
+#pragma unroll
+          for (int s = 1; s < NM; ++s) ys = s == sp ? y[s] : ys;
+          const double f = comb_factor<double>(ys, m);
+          v = k == 0 ? f : v * f;
+        }
+      }
+    } else {
+#pragma unroll
+      for (int s = 0; s < NM; ++s) {
+        const int m = md.ord[j][s];
+        if (m != 0) v = v * comb_factor<double>(y[s], m);
+      }
     }
     return v;
   }
@@ -343,12 +667,20 @@ struct ThreadTraj {
     return v;
   }
 
+  // The reaction that holds the integral G of reaction j: the lowest one with the same
+  // reactants, whose g, and so whose G, is the same number.  Known only where the tables are
+  // compiled in (gene expression: 4 integrals for 6 reactions); padded reactions have none.
+  __device__ static __forceinline__ constexpr int g_owner(int j) {
+    if constexpr (Model::kCompiled) return Model{}.gown[j];
+    else return j;
+  }
+
   __device__ static __forceinline__ void eval_props(const Model& md, const long long (&x)[NM],
                                                     const R (&th)[MM], R (&g)[MM], R (&a)[MM]) {
 #pragma unroll
     for (int j = 0; j < MM; ++j) {
       g[j] = g_int(md, j, x);
-      a[j] = th[j] * g[j];
+      a[j] = P::mul(th[j], g[j]);
     }
   }
 
@@ -366,17 +698,23 @@ struct ThreadTraj {
         for (int j = 0; j < MM; ++j) {
           const int v = md.nu[j][s];
           if (((use >> j) & 1u) && v != 0) {
-            mu = mu + (R)v * a[j];
-            var = var + (R)(v * v) * a[j];
+            if (P::kRef && (v == 1 || v == -1)) {  // the products are exact
+              mu = v > 0 ? mu + a[j] : mu - a[j];
+              var = var + a[j];
+            } else {
+              mu = P::mad((R)v, a[j], mu);
+              var = P::mad((R)(v * v), a[j], var);
+            }
           }
         }
         const R h = hor_factor<R>(md.hor[s], x[s]);
-        R bound = (eps * (R)x[s]) / h;
-        if (bound < R(1)) bound = R(1);
+        R bound = eps * of_count<R>(x[s]);
+        if (md.hor[s] != kHorO1) bound = bound / h;  // h = 1 for a first-order reactant
+        if (P::lt(bound, R(1))) bound = R(1);
         const R t1 = bound / fabs(mu);
         const R t2 = (bound * bound) / var;
-        const R ts = t1 < t2 ? t1 : t2;
-        if (ts < tau) tau = ts;
+        const R ts = P::lt(t1, t2) ? t1 : t2;
+        if (P::lt(ts, tau)) tau = ts;
       }
     }
     return tau;
@@ -397,15 +735,16 @@ struct ThreadTraj {
     double c[NM];
 #pragma unroll
     for (int s = 0; s < NM; ++s) {
-      double acc = (double)x[s];
+      const double xs = f64_of_count(x[s]);
+      double acc = xs;
 #pragma unroll
       for (int j = 0; j < MM; ++j) {
         const int v = md.nu[j][s];
         if (((nc >> j) & 1u) && v != 0)
-          acc = acc + (double)v * ((double)Pk[j] - (double)a[j] * tau);
+          acc = acc + nu_times(v, f64_of_count(Pk[j]) - (double)a[j] * tau);
       }
       c[s] = acc;
-      y[s] = (double)x[s];
+      y[s] = xs;
     }
     const R taur = (R)tau;
     for (int it = 0; it < maxit; ++it) {
@@ -419,7 +758,7 @@ struct ThreadTraj {
 #pragma unroll
         for (int j = 0; j < MM; ++j) {
           const int v = md.nu[j][s];
-          if (((nc >> j) & 1u) && v != 0) acc = acc + (double)v * ay[j];
+          if (((nc >> j) & 1u) && v != 0) acc = acc + nu_times(v, ay[j]);
         }
         b[s] = (R)(-((y[s] - c[s]) - tau * acc));
       }
@@ -455,7 +794,8 @@ struct ThreadTraj {
 #pragma unroll
           for (int j = 0; j < MM; ++j) {
             const int v = md.nu[j][s];
-            if (((nc >> j) & 1u) && v != 0 && md.ord[j][q] != 0) acc = acc + (R)v * Dq[j];
+            if (((nc >> j) & 1u) && v != 0 && md.ord[j][q] != 0)
+              acc = acc + nu_times(v, Dq[j]);
           }
           A[s][q] = (s == q ? R(1) : R(0)) - taur * acc;
         }
@@ -467,12 +807,12 @@ struct ThreadTraj {
         R best = fabs(A[k][k]);
 #pragma unroll
         for (int i = k + 1; i < NM; ++i) {
-          if (fabs(A[i][k]) > best) {
+          if (abs_gt(A[i][k], best)) {
             best = fabs(A[i][k]);
             piv = i;
           }
         }
-        if (best == R(0)) return 2;
+        if (P::zero(best)) return 2;
 #pragma unroll
         for (int i = k + 1; i < NM; ++i) {
           if (i == piv) {
@@ -666,18 +1006,78 @@ struct ThreadTraj {
   // of block w (words 2, 3).  Reference: sequential prefix sums in index order (the
   // canonical order), target u * sum with the lane-tree sum.  Fast: see pick_fast.
   // Rounding that leaves no hit picks the last positive entry.
-  __device__ static __forceinline__ int pick_reaction(const R (&v)[MM], const Words4& w) {
-    if (!P::kRef) return pick_fast(v, w);
+  // tot: the lane-tree sum of v (reference precision).
+  __device__ static __forceinline__ int pick_reaction(const R (&v)[MM], const Words4& w,
+                                                      R tot) {
+    if constexpr (!P::kRef) {
+      return pick_fast(v, w);
+    } else {
+      bool clear;
+      const int pk = pick_near(v, w, clear);
+      return clear ? pk : pick_ref(v, w, tot);
+    }
+  }
+
+  // Reference precision's pick, first in FP32 on truncated values: they are off by 2^-23
+  // relative, each of the M sums by 2^-24, so prefixes and total lie within (M + 2) 2^-24
+  // tot of the FP64 ones (themselves within M 2^-53 tot of exact) and the target, with the
+  // uniform's upper 24 bits, within (M + 5) 2^-24 tot; when the target is farther than
+  // (M + 4) 2^-23 tot from every prefix the FP64 search gives the same reaction.  Otherwise
+  // (about 1e-5 of the picks), and when the total is outside FP32's middle range, the FP64
+  // search has to run: M additions, a product and comparisons on the FP64 unit.
+  __device__ static __forceinline__ int pick_near(const R (&v)[MM], const Words4& w,
+                                                  bool& clear) {
+    float pre[MM];
+    float acc = 0.f;
+#pragma unroll
+    for (int j = 0; j < MM; ++j) {
+      acc = acc + f32_near((double)v[j]);
+      pre[j] = acc;
+    }
+    const int pk = search_prefix(pre, w.w2, MM + 4, clear);
+    clear = clear && acc > 0x1p-60f && acc < 0x1p60f;
+    return pk;
+  }
+
+  // An FP64 value in [0, 2^127) as FP32 within 2^-23 relative (truncated; below the FP32
+  // normal range 0; beyond it infinity, which the caller's range test catches).
+  __device__ static __forceinline__ float f32_near(double d) {
+    const uint32_t hi = (uint32_t)__double2hiint(d), lo = (uint32_t)__double2loint(d);
+    if (hi < 0x38100000u) return 0.f;
+    if (hi >= 0x47e00000u) return inf32();
+    return __uint_as_float(((hi - 0x38000000u) << 3) | (lo >> 29));
+  }
+  __device__ static __forceinline__ float inf32() { return __int_as_float(0x7f800000); }
+
+  __device__ static __noinline__ int pick_ref(const R (&v)[MM], const Words4& w, R tot) {
     int pk = -1, last = -1;
-    const R target = P::u(w, 1) * lane_tree_sum<MM, R>(v);
+    const R target = P::u(w, 1) * tot;
     R acc = R(0);
 #pragma unroll
     for (int j = 0; j < MM; ++j) {
-      if (v[j] > R(0)) last = j;
+      if (P::positive(v[j])) last = j;
       acc = acc + v[j];
-      if (pk < 0 && target < acc) pk = j;
+      if (pk < 0 && P::lt(target, acc)) pk = j;
     }
     return pk < 0 ? last : pk;
+  }
+
+  // The reaction whose prefix interval holds the target, by FP32 prefix sums `pre` (the
+  // last one the total) and the upper 24 bits of the uniform; clear = the target is farther
+  // than `ulps` 2^-23 of the total from every prefix.
+  __device__ static __forceinline__ int search_prefix(const float (&pre)[MM], uint32_t w2,
+                                                      int ulps, bool& clear) {
+    const float target = (float)(w2 >> 8) * 0x1p-24f * pre[MM - 1];
+    const float margin = (float)ulps * 0x1p-23f * pre[MM - 1];
+    int pk = 0;
+    float near = inf32();
+#pragma unroll
+    for (int j = 0; j < MM; ++j) {
+      pk += pre[j] <= target ? 1 : 0;
+      near = fminf(near, fabsf(pre[j] - target));
+    }
+    clear = near > margin && pk < MM;
+    return pk;
   }
 
   // Fast precision pick with a 48-bit uniform u = (w2>>8) 2^-24 + ((w3>>8) + 1/2) 2^-48.
@@ -695,17 +1095,9 @@ struct ThreadTraj {
       acc = acc + (float)v[j];
       pre[j] = acc;
     }
-    const float target = (float)(w.w2 >> 8) * 0x1p-24f * acc;
-    const float margin = (float)(MM + 2) * 0x1p-23f * acc;
-    int pk = 0;
-    bool clear = true;
-#pragma unroll
-    for (int j = 0; j < MM; ++j) {
-      pk += pre[j] <= target ? 1 : 0;
-      clear = clear && fabsf(pre[j] - target) > margin;
-    }
-    if (clear && pk < MM) return pk;
-    return pick_df(v, w);
+    bool clear;
+    const int pk = search_prefix(pre, w.w2, MM + 2, clear);
+    return clear ? pk : pick_df(v, w);
   }
 
   // The same search over double-float (TwoSum) prefix sums of the FP32 values with the
@@ -758,19 +1150,20 @@ __device__ __noinline__ int implicit_leap_wide(const MDL& md,
   double th[MM], ax[MM], y[NM], c[NM];
 #pragma unroll
   for (int j = 0; j < MM; ++j) {
-    th[j] = (double)io.th[j];
+    th[j] = f64_of_f32(io.th[j]);
     ax[j] = th[j] * TR::g_int(md, j, io.x);
   }
 #pragma unroll
   for (int s = 0; s < NM; ++s) {
-    double acc = (double)io.x[s];
+    const double xs = f64_of_count(io.x[s]);
+    double acc = xs;
 #pragma unroll
     for (int j = 0; j < MM; ++j) {
       const int v = md.nu[j][s];
-      if (((nc >> j) & 1u) && v != 0) acc += (double)v * ((double)io.K[j] - ax[j] * tau);
+      if (((nc >> j) & 1u) && v != 0) acc += nu_times(v, f64_of_count(io.K[j]) - ax[j] * tau);
     }
     c[s] = acc;
-    y[s] = (double)io.x[s];
+    y[s] = xs;
   }
   int rc = 1;
   for (int it = 0; it < maxit && rc == 1; ++it) {
@@ -784,7 +1177,7 @@ __device__ __noinline__ int implicit_leap_wide(const MDL& md,
 #pragma unroll
       for (int j = 0; j < MM; ++j) {
         const int v = md.nu[j][s];
-        if (v != 0) acc += (double)v * ay[j];
+        if (v != 0) acc += nu_times(v, ay[j]);
       }
       b[s] = -((y[s] - c[s]) - tau * acc);
     }
@@ -816,7 +1209,7 @@ __device__ __noinline__ int implicit_leap_wide(const MDL& md,
 #pragma unroll
         for (int j = 0; j < MM; ++j) {
           const int v = md.nu[j][s];
-          if (v != 0 && md.ord[j][q] != 0) acc += (double)v * Dq[j];
+          if (v != 0 && md.ord[j][q] != 0) acc += nu_times(v, Dq[j]);
         }
         A[s][q] = (s == q ? 1.0 : 0.0) - tau * acc;
       }
@@ -828,12 +1221,12 @@ __device__ __noinline__ int implicit_leap_wide(const MDL& md,
       double best = fabs(A[k][k]);
 #pragma unroll
       for (int i = k + 1; i < NM; ++i) {
-        if (fabs(A[i][k]) > best) {
+        if (f64_abs_gt(A[i][k], best)) {
           best = fabs(A[i][k]);
           piv = i;
         }
       }
-      if (!(best > 0.0)) {
+      if (!f64_abs_gt(best, 0.0)) {
         rc = 2;
         break;
       }
@@ -920,8 +1313,12 @@ __device__ __noinline__ int implicit_leap_fp32(const MDL& md,
 // kernels).
 // kGrid: time-grid output compiled in.  Without it the grid code is absent, so the
 // kernels that serve calls without a grid are exactly the plain simulation.
+constexpr int kSsaPerRound = 8;  // firings of a slice
+constexpr int kUnit = 4;         // firings done together without a branch
+
 template <int NM, int MM, class P, bool kGrid = false, class MDL = ThreadModel<NM, MM>>
 struct ThreadLane {
+  static_assert(kSsaPerRound < 16 && MM <= 16, "a slice's firings are 4 bits per reaction");
   using R = typename P::R;
   using TT = ThreadTraj<NM, MM, P, MDL>;
   using Model = MDL;
@@ -977,7 +1374,10 @@ struct ThreadLane {
       status |= ML_ST_BAD_INPUT;
       t = T;
     }
-    if (T != T) t = 0.0;  // NaN horizon: finishes at once
+    if (T != T) {  // NaN horizon: finishes at once
+      t = 0.0;
+      T = -1.0;
+    }
     mode = kEval;
     if (kGrid && A.K_obs > 0) record(A, t, true);  // grid points at t = 0 see x0
   }
@@ -1035,7 +1435,7 @@ struct ThreadLane {
     for (int j = 0; j < MM; ++j) {
       if (j < A.M) {
         A.r[i * A.M + j] = r[j];
-        A.G[i * A.M + j] = G[j];
+        A.G[i * A.M + j] = G[TT::g_owner(j)];
       }
     }
     A.status[i] = status | (staged ? 0u : ML_ST_STAGE_TIMEOUT);
@@ -1049,8 +1449,14 @@ struct ThreadLane {
   // The lane state as 32-bit words of a shared-memory record (pool driver): word k of
   // slot q at rec[k * kPoolSlots + q], the mode first.  g, a and a0 are not kept: a
   // loaded lane recomputes them from x and theta before use.
+  template <class MD>
+  __device__ static constexpr int g_owner_count() {
+    if constexpr (MD::kCompiled) return MD::n_gown;
+    else return MM;
+  }
   static constexpr int kRWords = (int)(sizeof(R) / 4);
-  static constexpr int kWords = lane_record_words(NM, MM, kRWords == 2);
+  static constexpr int kWords =
+      lane_record_words(NM, MM, kRWords == 2) - 2 * (MM - g_owner_count<Model>());
   template <int S>
   __device__ __forceinline__ void save(uint32_t* rec, int q) const {
     int k = 0;
@@ -1079,7 +1485,8 @@ struct ThreadLane {
 #pragma unroll
     for (int j = 0; j < MM; ++j) put64((unsigned long long)r[j]);
 #pragma unroll
-    for (int j = 0; j < MM; ++j) put64((unsigned long long)__double_as_longlong(G[j]));
+    for (int j = 0; j < MM; ++j)
+      if (TT::g_owner(j) == j) put64((unsigned long long)__double_as_longlong(G[j]));
 #pragma unroll
     for (int c = 0; c < 4; ++c) put64((unsigned long long)cnt[c]);
   }
@@ -1111,7 +1518,8 @@ struct ThreadLane {
 #pragma unroll
     for (int j = 0; j < MM; ++j) r[j] = (long long)get64();
 #pragma unroll
-    for (int j = 0; j < MM; ++j) G[j] = __longlong_as_double((long long)get64());
+    for (int j = 0; j < MM; ++j)
+      if (TT::g_owner(j) == j) G[j] = __longlong_as_double((long long)get64());
 #pragma unroll
     for (int c = 0; c < 4; ++c) cnt[c] = (long long)get64();
   }
@@ -1128,132 +1536,262 @@ struct ThreadLane {
     mode = kEval;
   }
 
-  // Up to n_slice firings of the SSA burst (Gillespie 1977 direct method) at outer step
-  // `step`, firing index b; g, a, a0 are current for b == 0 (or recomputed with fresh).
-  // Fast precision accumulates the slice's G increments in FP32 and its elapsed time in
-  // compensated FP32 and folds them into the FP64 totals at the end of the slice (every
-  // driver runs slices of kSsaPerRound firings, so all fold at the same firings).  The firing counts of the slice are kept in
-  // 32-bit registers and added to r once at the end.  The random block of the next
-  // firing is generated while the current one is processed: it depends only on the
-  // counter, so the two dependency chains overlap.
-  __device__ __forceinline__ void ssa_slice(const Model& md, const SimArgs& A, int n_slice,
-                                            bool fresh = false) {
-    const uint32_t k0 = (uint32_t)A.seed, k1 = (uint32_t)(A.seed >> 32);
-    const uint32_t Mr = (uint32_t)A.M;
-    const double rem = T - t;
-    const float remf = (float)rem;
-    float el = 0.f, elc = 0.f;
-    float Gs[MM];
-    int rc[MM];
+  // Adds v to the integral of every reaction that holds one.
+  template <class F>
+  __device__ __forceinline__ void add_G(F v) {
 #pragma unroll
-    for (int j = 0; j < MM; ++j) {
-      Gs[j] = 0.f;
-      rc[j] = 0;
-    }
-    // fast precision: an FP32 copy of the state, updated with the FP32 net changes, so
-    // that the propensities need no 64-bit conversions; synchronized at every slice start
-    float xf[NM];
+    for (int j = 0; j < MM; ++j)
+      if (TT::g_owner(j) == j) G[j] = G[j] + v(j);
+  }
+
+  // The net changes of reaction `pick` on the FP32 state copy / on the counts.
+  __device__ __forceinline__ static void fire_f(const Model& md, int pick, float (&xf)[NM]) {
+    if constexpr (Model::kCompiled) {  // one predicated update per nonzero entry
 #pragma unroll
-    for (int s = 0; s < NM; ++s) xf[s] = P::kRef ? 0.f : (float)x[s];
-    const int b_first = b;
-    bool to_horizon = false, burst_over = false;
-    Words4 w = philox_block(k0, k1, id, step, Mr + 2u, (uint32_t)b);
-    for (int k = 0; k < n_slice; ++k) {
-      if (b > 0 || (fresh && k == 0)) {  // the state changed at the previous firing
-        if (P::kRef) {
-          TT::eval_props(md, x, th, g, a);
-        } else {
+      for (int j = 0; j < MM; ++j) {
 #pragma unroll
-          for (int j = 0; j < MM; ++j) {
-            g[j] = (R)TT::g_flt(md, j, xf);
-            a[j] = th[j] * g[j];
-          }
-        }
-        a0 = reaction_sum<MM, R, P::kRef>(a);
-      }
-      if (a0 == R(0)) {
-        to_horizon = burst_over = true;
-        break;
-      }
-      const Words4 w_next = philox_block(k0, k1, id, step, Mr + 2u, (uint32_t)b + 1u);
-      if (P::kRef) {
-        const R dt = -P::log(P::u(w, 0)) / a0;
-        const double tn = t + (double)dt;
-        if (tn > T) {
-          to_horizon = burst_over = true;
-          break;
-        }
-#pragma unroll
-        for (int j = 0; j < MM; ++j) G[j] = G[j] + (double)g[j] * (double)dt;
-        if (kGrid && A.K_obs > 0) record(A, tn, false);  // points before the firing: old state
-        t = tn;
-      } else {
-        const float dt = __fdividef(-P::log(P::u(w, 0)), a0);  // about 2 ulp
-        if ((el - elc) + dt > remf) {
-          to_horizon = burst_over = true;
-          break;
-        }
-        // a slice holds at most kSsaPerRound firings: its G sums of that many positive
-        // terms are within 8 FP32 roundings; the elapsed time is summed compensated
-#pragma unroll
-        for (int j = 0; j < MM; ++j) Gs[j] = fmaf((float)g[j], dt, Gs[j]);
-        kahan_add(el, elc, dt);
-        if (kGrid && A.K_obs > 0) record(A, t + ((double)el - (double)elc), false);
-      }
-      const int pick = TT::pick_reaction(a, w);
-      if constexpr (Model::kCompiled) {
-        // compile-time net changes: one predicated update per nonzero entry
-#pragma unroll
-        for (int j = 0; j < MM; ++j) {
-#pragma unroll
-          for (int s = 0; s < NM; ++s) {
-            if (md.nu[j][s] != 0 && j == pick) {
-              x[s] += md.nu[j][s];
-              if (!P::kRef) xf[s] += md.nuf[j][s];
-            }
-          }
-        }
-      } else {
-#pragma unroll
-        for (int s = 0; s < NM; ++s) {
-          x[s] += md.nu[pick][s];
-          if (!P::kRef) xf[s] += md.nuf[pick][s];
-        }
-      }
-#pragma unroll
-      for (int j = 0; j < MM; ++j) rc[j] += (j == pick) ? 1 : 0;
-      if (kGrid && A.K_obs > 0)  // a point at the firing time: new state
-        record(A, P::kRef ? t : t + ((double)el - (double)elc), true);
-      w = w_next;
-      if (++b >= n_max) {
-        burst_over = true;
-        break;
-      }
-    }
-#pragma unroll
-    for (int j = 0; j < MM; ++j) r[j] += rc[j];
-    cnt[2] += b - b_first;
-    if (P::kRef) {
-      if (to_horizon) {
-        const double rm = T - t;
-#pragma unroll
-        for (int j = 0; j < MM; ++j) G[j] = G[j] + (double)g[j] * rm;
-        t = T;
+        for (int s = 0; s < NM; ++s)
+          if (md.nu[j][s] != 0 && j == pick) xf[s] += md.nuf[j][s];
       }
     } else {
-      const double elapsed = (double)el - (double)elc;
-      // one FP64 addition per reaction and slice
 #pragma unroll
-      for (int j = 0; j < MM; ++j) G[j] = G[j] + (double)Gs[j];
-      if (to_horizon) {
-        const double left = rem - elapsed > 0.0 ? rem - elapsed : 0.0;
-#pragma unroll
-        for (int j = 0; j < MM; ++j) G[j] = G[j] + (double)g[j] * left;
-        t = T;
-      } else {
-        t = t + elapsed;
-      }
+      for (int s = 0; s < NM; ++s) xf[s] += md.nuf[pick][s];
     }
+  }
+  __device__ __forceinline__ static void fire_x(const Model& md, int pick, long long (&x)[NM]) {
+    if constexpr (Model::kCompiled) {
+#pragma unroll
+      for (int j = 0; j < MM; ++j) {
+#pragma unroll
+        for (int s = 0; s < NM; ++s)
+          if (md.nu[j][s] != 0 && j == pick) x[s] += md.nu[j][s];
+      }
+    } else {
+#pragma unroll
+      for (int s = 0; s < NM; ++s) x[s] += md.nu[pick][s];
+    }
+  }
+  // ... and of the firings counted in the nibbles of `fired`.
+  __device__ __forceinline__ void fold_x(const Model& md, unsigned long long fired) {
+#pragma unroll
+    for (int j = 0; j < MM; ++j) {
+      const int c = (int)(fired >> (4 * j)) & 15;
+#pragma unroll
+      for (int s = 0; s < NM; ++s) x[s] += (long long)((int)md.nu[j][s] * c);
+    }
+  }
+
+  // A slice's running sums: elapsed time (compensated FP32), G increments, the FP32 copy
+  // of the state, and the firings, 4 bits per reaction.
+  struct Slice {
+    float el, elc;
+    float Gs[MM], xf[NM];
+    unsigned long long fired;
+  };
+
+  // kUnit firings without a branch: their random blocks, waiting times' logarithms and
+  // uniforms first (independent of each other and of the state, so their chains overlap),
+  // then the firings, each with its choices as selects.  Nothing is committed (false) when
+  // one of them needs more: no reaction possible, the horizon or (kGrid) an observation
+  // point reached, or a pick too near a prefix for FP32; the careful loop of ssa_slices
+  // then does them one by one.  A lane spends most of its time here, and with few warps per
+  // scheduler the chains' latency decides: one firing at a time, with its four branches,
+  // took about 1,300 cycles on the immigration-death batch of 10,000 (one warp per
+  // scheduler), most of it waiting for the ten rounds of Philox and the logarithm.
+  __device__ __forceinline__ bool unit(const Model& md, const SimArgs& A, Slice& sl,
+                                       float remf) {
+    const uint32_t k0 = (uint32_t)A.seed, k1 = (uint32_t)(A.seed >> 32);
+    R wait[kUnit];
+    Words4 w[kUnit];
+#pragma unroll
+    for (int i = 0; i < kUnit; ++i) {
+      w[i] = philox_block(k0, k1, id, step, (uint32_t)A.M + 2u, (uint32_t)b + (uint32_t)i);
+      wait[i] = -P::log(P::u(w[i], 0));
+    }
+    bool ok = true;
+    if constexpr (P::kRef) {
+      double tn = t, Gn[MM];
+      long long xn[NM];
+#pragma unroll
+      for (int j = 0; j < MM; ++j) Gn[j] = G[j];
+#pragma unroll
+      for (int s = 0; s < NM; ++s) xn[s] = x[s];
+      unsigned long long fired = sl.fired;
+#pragma unroll
+      for (int i = 0; i < kUnit; ++i) {
+        TT::eval_props(md, xn, th, g, a);
+        a0 = reaction_sum<MM, R, P::kRef>(a);
+        const double dt = wait[i] / a0;
+        tn = tn + dt;
+        ok = ok && P::positive(a0) && !f64_lt_nn(T, tn);
+#pragma unroll
+        for (int j = 0; j < MM; ++j)
+          if (TT::g_owner(j) == j) Gn[j] = Gn[j] + (double)g[j] * dt;
+        bool clear;
+        const int pick = TT::pick_near(a, w[i], clear);
+        ok = ok && clear;
+        if (!ok) return false;
+        fire_x(md, pick, xn);
+        fired += 1ULL << (4 * pick);
+      }
+      if (kGrid && kobs < A.K_obs && !(__ldg(A.t_obs + kobs) > tn)) return false;
+      t = tn;
+#pragma unroll
+      for (int j = 0; j < MM; ++j) G[j] = Gn[j];
+#pragma unroll
+      for (int s = 0; s < NM; ++s) x[s] = xn[s];
+      sl.fired = fired;
+    } else {
+      Slice n = sl;
+      if (kGrid) n.fired = 0;
+#pragma unroll
+      for (int i = 0; i < kUnit; ++i) {
+        float pre[MM];
+        props_f(md, n.xf, pre);
+        const float dt = __fdividef(wait[i], pre[MM - 1]);  // about 2 ulp
+        ok = ok && pre[MM - 1] > 0.f && !((n.el - n.elc) + dt > remf);
+#pragma unroll
+        for (int j = 0; j < MM; ++j)
+          if (TT::g_owner(j) == j) n.Gs[j] = fmaf((float)g[j], dt, n.Gs[j]);
+        kahan_add(n.el, n.elc, dt);
+        bool clear;
+        int pick = TT::search_prefix(pre, w[i].w2, MM + 2, clear);
+        ok = ok && clear;
+        pick = pick < MM ? pick : 0;
+        fire_f(md, pick, n.xf);
+        n.fired += 1ULL << (4 * pick);
+      }
+      if (kGrid && kobs < A.K_obs &&
+          !(__ldg(A.t_obs + kobs) > t + ((double)n.el - (double)n.elc)))
+        return false;
+      if (!ok) return false;
+      if (kGrid) {
+        fold_x(md, n.fired);
+        n.fired += sl.fired;
+      }
+      sl = n;
+    }
+    b += kUnit;
+    return true;
+  }
+
+  // Fast precision: g and a from the FP32 state copy, and the prefix sums of a, whose last
+  // is the sequential total.
+  __device__ __forceinline__ void props_f(const Model& md, const float (&xf)[NM],
+                                          float (&pre)[MM]) {
+#pragma unroll
+    for (int j = 0; j < MM; ++j) {
+      g[j] = (R)TT::g_flt(md, j, xf);
+      a[j] = P::mul(th[j], g[j]);
+      pre[j] = j == 0 ? (float)a[0] : __fadd_rn(pre[j - 1], (float)a[j]);
+    }
+  }
+
+  // Up to n_slices slices of kSsaPerRound firings of the SSA burst (Gillespie 1977 direct
+  // method) at outer step `step`, firing index b.
+  // Fast precision accumulates a slice's G increments in FP32 and its elapsed time in
+  // compensated FP32 and folds them into the FP64 totals at the end of the slice: one FP64
+  // addition per integral, its operand widened on the integer pipe (every driver folds at
+  // the same firings).  The propensities read an FP32 copy of the state that the firings
+  // update; x and r take the slice's firings at its end.
+  // kUnits: firings in units, for the drivers whose few warps wait on the latency of a
+  // firing; the pool driver, bound by instruction fetch and issue, is slower with the larger
+  // loop (1,000,000 gene-expression trajectories: 375 ms against 300).
+  template <bool kUnits>
+  __device__ __forceinline__ void ssa_slices(const Model& md, const SimArgs& A, int n_slices) {
+    const uint32_t k0 = (uint32_t)A.seed, k1 = (uint32_t)(A.seed >> 32);
+    const int b_first = b;
+    bool burst_over = false;
+    for (;;) {
+      const double rem = P::kRef ? 0.0 : T - t;
+      const float remf = P::kRef ? 0.f : f32_of_f64(rem);
+      Slice sl;
+      sl.el = sl.elc = 0.f;
+      sl.fired = 0;
+#pragma unroll
+      for (int j = 0; j < MM; ++j) sl.Gs[j] = 0.f;
+      // an FP32 copy of the state, synchronized at every slice start
+#pragma unroll
+      for (int s = 0; s < NM; ++s) sl.xf[s] = P::kRef ? 0.f : f32_of_count(x[s]);
+      bool to_horizon = false;
+      const int b_end = b + kSsaPerRound < n_max ? b + kSsaPerRound : n_max;
+#pragma unroll 1
+      while (b < b_end && !burst_over) {
+        if constexpr (kUnits && (Model::kCompiled || MM <= 2))
+          if (b + kUnit <= b_end && unit(md, A, sl, remf)) continue;
+        // one by one
+        const int b_stop = b + kUnit < b_end ? b + kUnit : b_end;
+#pragma unroll 1
+        for (; b < b_stop; ++b) {
+          if constexpr (P::kRef) {
+            TT::eval_props(md, x, th, g, a);
+            a0 = reaction_sum<MM, R, P::kRef>(a);
+          } else {
+            float pre[MM];
+            props_f(md, sl.xf, pre);
+            a0 = (R)pre[MM - 1];
+          }
+          if (P::zero(a0)) {
+            to_horizon = burst_over = true;
+            break;
+          }
+          const Words4 w = philox_block(k0, k1, id, step, (uint32_t)A.M + 2u, (uint32_t)b);
+          if constexpr (P::kRef) {
+            const R dt = -P::log(P::u(w, 0)) / a0;
+            const double tn = t + (double)dt;
+            if (f64_lt_nn(T, tn)) {
+              to_horizon = burst_over = true;
+              break;
+            }
+            add_G([&](int j) { return (double)g[j] * (double)dt; });
+            if (kGrid && A.K_obs > 0) record(A, tn, false);  // points before the firing: old state
+            t = tn;
+          } else {
+            const float dt = __fdividef(-P::log(P::u(w, 0)), a0);
+            if ((sl.el - sl.elc) + dt > remf) {
+              to_horizon = burst_over = true;
+              break;
+            }
+            // a slice holds at most kSsaPerRound firings: its G sums of that many positive
+            // terms are within 8 FP32 roundings; the elapsed time is summed compensated
+#pragma unroll
+            for (int j = 0; j < MM; ++j)
+              if (TT::g_owner(j) == j) sl.Gs[j] = fmaf((float)g[j], dt, sl.Gs[j]);
+            kahan_add(sl.el, sl.elc, dt);
+            if (kGrid && A.K_obs > 0) record(A, t + ((double)sl.el - (double)sl.elc), false);
+          }
+          const int pick = TT::pick_reaction(a, w, a0);
+          if (P::kRef || kGrid) fire_x(md, pick, x);
+          if (!P::kRef) fire_f(md, pick, sl.xf);
+          sl.fired += 1ULL << (4 * pick);
+          if (kGrid && A.K_obs > 0)  // a point at the firing time: new state
+            record(A, P::kRef ? t : t + ((double)sl.el - (double)sl.elc), true);
+        }
+      }
+      if (b >= n_max) burst_over = true;
+#pragma unroll
+      for (int j = 0; j < MM; ++j) r[j] += (int)(sl.fired >> (4 * j)) & 15;
+      if (!P::kRef && !kGrid) fold_x(md, sl.fired);
+      if constexpr (P::kRef) {
+        if (to_horizon) {
+          const double rm = T - t;
+          add_G([&](int j) { return (double)g[j] * rm; });
+          t = T;
+        }
+      } else {
+        const double elapsed = f64_of_f32(sl.el) - f64_of_f32(sl.elc);
+        add_G([&](int j) { return f64_of_f32(sl.Gs[j]); });
+        if (to_horizon) {
+          const double left = rem - elapsed > 0.0 ? rem - elapsed : 0.0;
+          add_G([&](int j) { return (double)g[j] * left; });
+          t = T;
+        } else {
+          t = t + elapsed;
+        }
+      }
+      if (burst_over || --n_slices <= 0) break;
+    }
+    cnt[2] += b - b_first;
     if (burst_over) end_burst();
   }
 
@@ -1262,7 +1800,7 @@ struct ThreadLane {
   __device__ __forceinline__ void eval_phase(const Model& md, const SimArgs& A) {
     const uint32_t k0 = (uint32_t)A.seed, k1 = (uint32_t)(A.seed >> 32);
     const uint32_t Mr = (uint32_t)A.M;  // stream numbering uses the real M
-    if (!(t < T)) {
+    if (!f64_lt_nn(t, T)) {
       mode = kDone;
       return;
     }
@@ -1285,16 +1823,15 @@ struct ThreadLane {
     }
     TT::eval_props(md, x, th, g, a);
     a0 = reaction_sum<MM, R, P::kRef>(a);
-    if (a0 == R(0)) {
+    if (P::zero(a0)) {
       const double rm = T - t;
-#pragma unroll
-      for (int j = 0; j < MM; ++j) G[j] = G[j] + (double)g[j] * rm;
+      add_G([&](int j) { return (double)g[j] * rm; });
       t = T;
       mode = kDone;
       return;
     }
     int burst = 0;
-    const R eps = (R)A.eps;
+    const R eps = P::eps(A);
     if (A.mode == ML_MODE_SSA_ONLY) {
       burst = A.n_ssa_ex;
     } else {
@@ -1305,7 +1842,7 @@ struct ThreadLane {
 #pragma unroll
       for (int j = 0; j < MM; ++j) {
         bool crit = false;
-        if (a[j] > R(0)) {
+        if (P::positive(a[j])) {
 #pragma unroll
           for (int s = 0; s < NM; ++s) {
             const int v = md.nu[j][s];
@@ -1330,13 +1867,13 @@ struct ThreadLane {
 #pragma unroll
             for (int kk = 0; kk < MM; ++kk)
               if (kk == k) ak = a[kk];
-            const R lo = a[j] < ak ? a[j] : ak;
-            if (fabs(a[j] - ak) <= (R)A.pe_delta * lo) pe |= (1u << j) | (1u << k);
+            const R lo = P::lt(a[j], ak) ? a[j] : ak;
+            if (!P::lt(P::pe_delta(A) * lo, fabs(a[j] - ak))) pe |= (1u << j) | (1u << k);
           }
         }
         if (pe != 0) {
           const R tau_im = TT::tau_select(md, a, x, nc & ~pe, eps);
-          if (tau_im > (R)A.stiff_ratio * tau_ex) {
+          if (P::lt(P::stiff_ratio(A) * tau_ex, tau_im)) {
             implicit = true;
             tau1 = tau_im;
           }
@@ -1350,30 +1887,31 @@ struct ThreadLane {
           break;
         }
         R tau2 = P::inf();
-        if (a0c > R(0)) {
+        if (P::positive(a0c)) {
           const Words4 w = philox_block(k0, k1, id, step, Mr, 0u);
           tau2 = -P::log(P::u(w, 0)) / a0c;
         }
-        const R tmin = tau1 < tau2 ? tau1 : tau2;
-        if (tmin < (R)A.ssa_factor / a0) {
+        const R tmin = P::lt(tau1, tau2) ? tau1 : tau2;
+        if (P::lt(tmin, P::ssa_factor(A) / a0)) {
           burst = implicit ? A.n_ssa_im : A.n_ssa_ex;
           break;
         }
         const double stop = kGrid ? stop_time(A) : T;
         const double rm = stop - t;
         R tau = tau1;
-        if (tau2 < tau) tau = tau2;
+        if (P::lt(tau2, tau)) tau = tau2;
         bool at_horizon = false;
-        if ((R)rm <= tau) {
-          tau = (R)rm;
+        const R rmr = P::of_f64(rm);
+        if (!P::lt(tau, rmr)) {
+          tau = rmr;
           at_horizon = true;
         }
-        const bool crit_fire = (tau2 <= tau1) && (tau2 <= (R)rm);
+        const bool crit_fire = !P::lt(tau1, tau2) && !P::lt(rmr, tau2);
         {
           bool over = false;
 #pragma unroll
           for (int j = 0; j < MM; ++j)
-            over = over || (((nc >> j) & 1u) && a[j] * tau > (R)kLeapLimit);
+            over = over || (((nc >> j) & 1u) && P::lt((R)kLeapLimit, P::mul(a[j], tau)));
           if (over) {
             status |= ML_ST_OVERFLOW;
             mode = kDone;
@@ -1385,17 +1923,66 @@ struct ThreadLane {
         for (int j = 0; j < MM; ++j) K[j] = 0;
         if (crit_fire) {
           const Words4 w = philox_block(k0, k1, id, step, Mr + 1u, 0u);
-          const int pick = TT::pick_reaction(ac, Words4{0u, 0u, w.w0, w.w1});
+          const int pick = TT::pick_reaction(ac, Words4{0u, 0u, w.w0, w.w1}, a0c);
 #pragma unroll
           for (int j = 0; j < MM; ++j) K[j] = (j == pick) ? 1 : 0;
         }
-        const bool implicit_step = implicit && tau > tau_ex;
+        const bool implicit_step = implicit && P::lt(tau_ex, tau);
         // Poisson firings of the non-critical reactions (explicit counts, or the noise
         // term P_j of the implicit equation)
+        // The small means by inversion, reaction by reaction; the large ones by a loop over
+        // (reaction, PTRS trial) in which every lane is at a reaction of its own, so that the
+        // trial's code runs as often as the busiest lane needs it, not once per reaction that
+        // some lane of the warp draws by it.
+        // The first random block of every reaction is generated before any is used: their
+        // chains of ten dependent rounds (150 cycles each) overlap.
+        uint32_t big = 0;
+        R mus[MM];
+        long long drawn[MM];
+        Words4 first[MM];
 #pragma unroll
         for (int j = 0; j < MM; ++j)
-          if ((nc >> j) & 1u)
-            K[j] = poisson_draw<P>(a[j] * tau, k0, k1, id, step, (uint32_t)j, status);
+          if (MM <= 6 || j < A.M) first[j] = philox_block(k0, k1, id, step, (uint32_t)j, 0u);
+#pragma unroll
+        for (int j = 0; j < MM; ++j) {
+          mus[j] = P::mul(a[j], tau);
+          if (((nc >> j) & 1u) && P::positive(mus[j])) {
+            if (P::lt(mus[j], R(10))) K[j] = poisson_invert_at<P>(mus[j], P::u(first[j], 0));
+            else big |= 1u << j;
+          }
+        }
+        const uint32_t by_trials = big;
+        uint32_t trial = 0;
+        while (big != 0) {
+          const int j = __ffs((int)big) - 1;
+          const R mu = mus[j];
+          long long k = 0;
+          bool done;
+          if (!P::kRef && mu > R(4.0e6)) {
+            const PoissonDraw d =
+                poisson_ptrs<PrecWide>((double)mu, k0, k1, id, step, (uint32_t)j);
+            k = d.k;
+            status |= d.flags;
+            done = true;
+          } else {
+            const Words4 w = trial == 0u ? first[j]
+                                         : philox_block(k0, k1, id, step, (uint32_t)j, trial);
+            done = ptrs_trial<P>(mu, w, k);
+            if (++trial == (uint32_t)kPtrsMaxTrials && !done) {
+              k = (long long)floor(mu + R(0.5));
+              status |= ML_ST_PTRS_CAP;
+              done = true;
+            }
+          }
+          if (done) {
+            drawn[j] = k;
+            big &= big - 1u;
+            trial = 0;
+          }
+        }
+#pragma unroll
+        for (int j = 0; j < MM; ++j)
+          if ((by_trials >> j) & 1u) K[j] = drawn[j];
         if (implicit_step) {
           int rc;
           if constexpr (P::kRef) {
@@ -1408,7 +1995,7 @@ struct ThreadLane {
               for (int j = 0; j < MM; ++j) {
                 if ((nc >> j) & 1u) {
                   const double ayj = (double)th[j] * TT::g_real(md, j, y);
-                  const double v = (ayj * taud + (double)K[j]) - (double)a[j] * taud;
+                  const double v = (ayj * taud + f64_of_count(K[j])) - (double)a[j] * taud;
                   const double rv = round(v);
                   K[j] = !(rv < 0x1p62) ? kCountLimit : (rv > 0.0 ? (long long)rv : 0);
                 }
@@ -1426,7 +2013,7 @@ struct ThreadLane {
             rc = A.newton_fp32
                      ? implicit_leap_fp32<NM, MM>(md, io, nc, (float)tau, A.newton_tol,
                                                   A.newton_maxit)
-                     : implicit_leap_wide<NM, MM>(md, io, nc, (double)tau, A.newton_tol,
+                     : implicit_leap_wide<NM, MM>(md, io, nc, P::to_f64(tau), A.newton_tol,
                                                   A.newton_maxit, A.fd_h,
                                                   A.jacobian == ML_JAC_ANALYTIC);
 #pragma unroll
@@ -1467,18 +2054,18 @@ struct ThreadLane {
           cnt[3] += 1;
           continue;
         }
-        const double half = (double)tau * 0.5;
         const R half_r = tau * R(0.5);
 #pragma unroll
         for (int j = 0; j < MM; ++j) {
-          const R gn = TT::g_int(md, j, xn);
           r[j] += K[j];
-          if (P::kRef) G[j] = G[j] + half * ((double)g[j] + (double)gn);
-          else G[j] = G[j] + (double)(half_r * (g[j] + gn));  // FP32 increment
+          if (TT::g_owner(j) == j) {  // fast precision: an FP32 increment
+            const R gn = TT::g_int(md, j, xn);
+            G[j] = G[j] + P::to_f64(half_r * (g[j] + gn));
+          }
         }
 #pragma unroll
         for (int s = 0; s < NM; ++s) x[s] = xn[s];
-        t = at_horizon ? stop : t + (double)tau;
+        t = at_horizon ? stop : t + P::to_f64(tau);
         if (kGrid && A.K_obs > 0) record(A, t, true);
         cnt[implicit_step ? 1 : 0] += 1;
         step++;
@@ -1505,7 +2092,14 @@ struct ThreadLane {
 // evaluation), so lanes in different phases progress together instead of a whole burst
 // holding the warp.  (Running only one phase per round, the evaluations once at least 4
 // or 8 lanes need one, measured 2.6 and 1.8 times slower on the gene-expression batch.)
-constexpr int kSsaPerRound = 8;
+// The first trajectory of a lane (n_traj: none): from the queue, or in the plain form by
+// position, per_warp of them to each warp.
+__device__ __forceinline__ long long first_index(const SimArgs& args, bool on) {
+  if (!on) return args.n_traj;
+  if (args.queue) return queue_claim(args.queue, args.order, args.n_traj);
+  const long long warp = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  return warp * args.per_warp + (threadIdx.x & 31);
+}
 
 // Round-based driver: plain form (queue null): thread i runs trajectory i.  Persistent
 // form: lanes claim trajectory indices from the device queue (in the caller's order, if
@@ -1515,8 +2109,8 @@ __device__ __forceinline__ void run_rounds(const MDL& md, bool staged, const Sim
   using Lane = ThreadLane<NM, MM, P, false, MDL>;
   Lane L;
   L.mode = Lane::kIdle;
-  const long long first = args.queue ? queue_claim(args.queue, args.order, args.n_traj)
-                                     : (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const bool on = (int)(threadIdx.x & 31) < args.per_warp;
+  const long long first = first_index(args, on);
   if (first < args.n_traj) L.start(md, args, first);
   for (;;) {
     if (L.mode == Lane::kDone) {
@@ -1530,7 +2124,7 @@ __device__ __forceinline__ void run_rounds(const MDL& md, bool staged, const Sim
     if (L.mode == Lane::kEval) {
       L.eval_phase(md, args);
     } else if (L.mode == Lane::kSsa) {
-      L.ssa_slice(md, args, kSsaPerRound);
+      L.template ssa_slices<true>(md, args, 1);
     }
   }
 }
@@ -1542,6 +2136,8 @@ __device__ __forceinline__ void run_rounds(const MDL& md, bool staged, const Sim
 // warp execute the same phase instead of taking turns between the evaluation and the SSA
 // code (the round-based driver's lanes diverge there).  A finished trajectory is written
 // out and its slot refilled from the work queue at once.  Persistent form only.
+
+constexpr int kPoolSlices = 13;  // slices of a visit: a burst of 100 firings to its end
 
 // Position of the (n+1)-th set bit of m (n < popcount(m)).
 __device__ __forceinline__ int nth_set_bit(unsigned long long m, int n) {
@@ -1563,7 +2159,8 @@ __device__ __forceinline__ void run_pool(const MDL& md, bool staged, const SimAr
   for (int h = lane; h < kPoolSlots; h += 32) {
     Lane L;
     L.mode = Lane::kIdle;
-    const long long idx = queue_claim(args.queue, args.order, args.n_traj);
+    const long long idx =
+        h < args.per_warp ? queue_claim(args.queue, args.order, args.n_traj) : args.n_traj;
     if (idx < args.n_traj) L.start(md, args, idx);
     L.template save<kPoolSlots>(rec, h);
   }
@@ -1591,7 +2188,7 @@ __device__ __forceinline__ void run_pool(const MDL& md, bool staged, const SimAr
       const int q = (nth_set_bit(mr, lane) + r0) & (kPoolSlots - 1);
       Lane L;
       L.template load<kPoolSlots>(rec, q);
-      if (ssa) L.ssa_slice(md, args, kSsaPerRound, true);
+      if (ssa) L.template ssa_slices<false>(md, args, kPoolSlices);
       else L.eval_phase(md, args);
       if (L.mode == Lane::kDone) {
         L.finish(args, staged);
@@ -1613,13 +2210,13 @@ template <int NM, int MM, class P, bool kGrid, class MDL>
 __device__ __forceinline__ void run_sequential(const MDL& md, bool staged, const SimArgs& args) {
   using Lane = ThreadLane<NM, MM, P, kGrid, MDL>;
   Lane L;
-  long long i = args.queue ? queue_claim(args.queue, args.order, args.n_traj)
-                           : (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const bool on = (int)(threadIdx.x & 31) < args.per_warp;
+  long long i = first_index(args, on);
   while (i < args.n_traj) {
     L.start(md, args, i);
     while (L.mode != Lane::kDone) {
       if (L.mode == Lane::kEval) L.eval_phase(md, args);
-      else L.ssa_slice(md, args, kSsaPerRound);
+      else L.template ssa_slices<true>(md, args, 1);
     }
     L.finish(args, staged);
     if (!args.queue) break;
