@@ -155,7 +155,7 @@ std::vector<uint8_t> warp_tables(const ml_model& m) {
   w.n_pairs = m.n_pairs;
   for (int j = 0; j < mlk::kWarpMaxM; ++j) {
     w.rates[j] = j < m.M ? m.rates[j] : 0.0;
-    w.partner[j] = -1;
+    w.pair[j] = -1;
     for (int q = 0; q < 3; ++q) w.rsp[j][q] = -1;
   }
   for (int j = 0; j < m.M; ++j) {
@@ -169,7 +169,7 @@ std::vector<uint8_t> warp_tables(const ml_model& m) {
       }
     }
     w.nreact[j] = (int8_t)q;
-    if (m.partner[j] > j) w.partner[j] = (int8_t)m.partner[j];
+    if (m.partner[j] >= 0) w.pair[j] = (int8_t)m.partner[j];
     uint64_t rm = 0, cm = 0;
     for (int s = 0; s < m.N; ++s) {
       if (m.ord[j * m.N + s] > 0) rm |= 1ULL << s;

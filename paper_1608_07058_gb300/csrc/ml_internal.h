@@ -84,7 +84,7 @@ struct alignas(16) WarpModel {
   int8_t rsp[kWarpMaxM][3];
   int8_t rmul[kWarpMaxM][3];
   int8_t nreact[kWarpMaxM];
-  int8_t partner[kWarpMaxM];      // as in ThreadModel
+  int8_t pair[kWarpMaxM];         // the other reaction of a reversible pair, else -1
   uint8_t isreact[kWarpMaxN];
   uint8_t hor[kWarpMaxN];
   // nonzero net changes of reaction j: rx_ptr[j] .. rx_ptr[j+1]

@@ -147,6 +147,14 @@ __device__ __forceinline__ void kahan_add(float& s, float& c, float v) {
 __device__ __forceinline__ bool lt_pos(double a, double b) { return f64_lt_pos(a, b); }
 __device__ __forceinline__ bool lt_pos(float a, float b) { return a < b; }
 
+// ... of the product a b, fused into the correction.
+__device__ __forceinline__ void kahan_fma(float& s, float& c, float a, float b) {
+  const float y = __fmaf_rn(a, b, -c);
+  const float t = s + y;
+  c = (t - s) - y;
+  s = t;
+}
+
 // Highest-order-reaction factor h_s (Cao 2006) from the species' flags and count.
 template <class R>
 __device__ __forceinline__ R hor_factor(uint8_t f, long long x) {

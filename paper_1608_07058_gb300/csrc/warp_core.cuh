@@ -74,6 +74,36 @@ __device__ inline WarpSlab carve_slab(char* p, int N, int M, int rbytes, int lby
   return s;
 }
 
+// Comparisons of the Newton system on the integer pipe: a > b for b >= -1 (a not negative;
+// false when a is NaN), equality of values that are not NaN, zero.
+__device__ __forceinline__ bool pivot_gt(double a, double b) {
+  const long long ua = __double_as_longlong(a);
+  return ua > __double_as_longlong(b) && ua <= 0x7ff0000000000000LL;
+}
+__device__ __forceinline__ bool pivot_gt(float a, float b) { return a > b; }
+__device__ __forceinline__ bool same_bits(double a, double b) {
+  return __double_as_longlong(a) == __double_as_longlong(b);
+}
+__device__ __forceinline__ bool same_bits(float a, float b) { return a == b; }
+__device__ __forceinline__ bool is_zero(double a) { return (__double_as_longlong(a) << 1) == 0; }
+__device__ __forceinline__ bool is_zero(float a) { return a == 0.f; }
+
+__device__ __forceinline__ double nu_as(int v, double) { return f64_of_i32(v); }
+__device__ __forceinline__ float nu_as(int v, float) { return (float)v; }
+
+// b / d rounded to nearest, given inv = 1 / d rounded to nearest (Markstein 1990: with the
+// rounded reciprocal and a quotient q within one unit in the last place, q + (b - q d) inv
+// rounds to the rounded quotient; the first correction brings b inv within that unit): five
+// FP64 instructions instead of nine.  Operands far from the ends of the exponent range.
+__device__ __forceinline__ double div_by_known(double b, double d, double inv) {
+  const int eb = (__double2hiint(b) >> 20) & 0x7ff, ed = (__double2hiint(d) >> 20) & 0x7ff;
+  if ((unsigned)(eb - 300) > 1400u || (unsigned)(ed - 800) > 400u) return b / d;
+  const double q = __dmul_rn(b, inv);
+  const double q1 = __fma_rn(__fma_rn(-d, q, b), inv, q);
+  return __fma_rn(__fma_rn(-d, q1, b), inv, q1);
+}
+__device__ __forceinline__ float div_by_known(float b, float d, float) { return b / d; }
+
 template <class P>
 struct WarpTraj {
   using R = typename P::R;
@@ -99,7 +129,7 @@ struct WarpTraj {
       const int s = md.rsp[j][k], m = md.rmul[j][k];
       const long long xs = x[s];
       if (xs < m) zero = true;
-      else v = v * comb_factor<R>((R)xs, m);
+      else v = v * comb_count<R>(xs, m);
     }
     return zero ? R(0) : v;
   }
@@ -133,10 +163,23 @@ struct WarpTraj {
   __device__ static __forceinline__ bool bit(const uint32_t (&m)[kRPL], int j) {
     return (m[j >> 5] >> (j & 31)) & 1u;
   }
+  // The bit of the lane's q-th own reaction.
+  __device__ static __forceinline__ bool own(const uint32_t (&m)[kRPL], int q, int lane) {
+    return (m[q] >> lane) & 1u;
+  }
 
-  // Cao 2006 step size over reactions in `use` (all lanes return the same value).
-  __device__ static R tau_select(const WarpModel& md, const R* a, const long long* x,
-                                 const uint32_t (&use)[kRPL], R eps, int lane) {
+  // Cao 2006 step size over the reactions whose bit in `use` is set (all lanes return the
+  // same value).  am: scratch for the propensities with the others' zeroed -- a zero leaves
+  // the sums as they are, and the lists need no test of a bit per entry.
+  __device__ static R tau_select(const WarpModel& md, const R (&a)[kRPL], R* am,
+                                 const long long* x, const uint32_t (&use)[kRPL], R eps,
+                                 int lane) {
+#pragma unroll
+    for (int q = 0; q < kRPL; ++q) {
+      const int j = lane + 32 * q;
+      if (j < md.M) am[j] = own(use, q, lane) ? a[q] : R(0);
+    }
+    __syncwarp();
     R tau = P::inf();
 #pragma unroll
     for (int q = 0; q < kSPL; ++q) {
@@ -144,27 +187,32 @@ struct WarpTraj {
       if (s < md.N && md.isreact[s]) {
         R mu = R(0), var = R(0);
         for (int e = md.sp_ptr[s]; e < md.sp_ptr[s + 1]; ++e) {
-          const int j = md.sp_j[e];
-          if (bit(use, j)) {
-            const int v = md.sp_nu[e];
-            mu = mu + (R)v * a[j];
-            var = var + (R)(v * v) * a[j];
+          const R aj = am[md.sp_j[e]];
+          const int v = md.sp_nu[e];
+          if (P::kRef && (v == 1 || v == -1)) {  // the products are exact
+            mu = v > 0 ? mu + aj : mu - aj;
+            var = var + aj;
+          } else {
+            mu = P::mad((R)v, aj, mu);
+            var = P::mad((R)(v * v), aj, var);
           }
         }
         const R h = hor_factor<R>(md.hor[s], x[s]);
-        R bound = (eps * (R)x[s]) / h;
-        if (bound < R(1)) bound = R(1);
+        R bound = eps * of_count<R>(x[s]);
+        if (md.hor[s] != kHorO1) bound = bound / h;  // h = 1 for a first-order reactant
+        if (P::lt(bound, R(1))) bound = R(1);
         const R t1 = bound / fabs(mu);
         const R t2 = (bound * bound) / var;
-        const R ts = t1 < t2 ? t1 : t2;
-        if (ts < tau) tau = ts;
+        const R ts = P::lt(t1, t2) ? t1 : t2;
+        if (P::lt(ts, tau)) tau = ts;
       }
     }
 #pragma unroll
     for (int d = 16; d >= 1; d >>= 1) {
       const R o = __shfl_xor_sync(0xffffffffu, tau, d);
-      tau = o < tau ? o : tau;
+      tau = P::lt(o, tau) ? o : tau;
     }
+    __syncwarp();
     return tau;
   }
 
@@ -177,15 +225,49 @@ struct WarpTraj {
   // same index.
   __device__ static int pick(const R* v, const R (&vl)[kRPL], const Words4& w, int M,
                              int lane) {
-    if (P::kRef) {
+    if constexpr (P::kRef) {
+      // First in FP32, on truncated values (2^-23 relative), summed by warp scans in index
+      // order (each sum within 2^-24 relative, at most 13 deep): prefixes and target are
+      // within 32 2^-24 of the total of the exact ones, the FP64 search within M 2^-53, so
+      // when the target is farther than 2^-18 of the total from every prefix both find the
+      // same reaction.  The FP64 search takes an addition and two comparisons per reaction
+      // on the FP64 unit, one after the other: 10,000 cycles for 100 reactions.
+      float pre[kRPL], tot = 0.f;
+#pragma unroll
+      for (int q = 0; q < kRPL; ++q) {
+        pre[q] = 0.f;
+        if (32 * q < M) {
+          float e = lane + 32 * q < M ? near32(vl[q]) : 0.f;
+#pragma unroll
+          for (int d = 1; d < 32; d <<= 1) {
+            const float o = __shfl_up_sync(0xffffffffu, e, d);
+            if (lane >= d) e = e + o;
+          }
+          pre[q] = tot + e;
+          tot = __shfl_sync(0xffffffffu, pre[q], 31);
+        }
+      }
+      const float near_t = (float)(w.w2 >> 8) * 0x1p-24f * tot, margin = 0x1p-18f * tot;
+      int found = -1;
+      bool clear = tot > 0x1p-60f && tot < 0x1p60f;
+#pragma unroll
+      for (int q = 0; q < kRPL; ++q) {
+        if (32 * q < M) {
+          const unsigned hit = __ballot_sync(0xffffffffu, near_t < pre[q] && lane + 32 * q < M);
+          if (found < 0 && hit) found = 32 * q + __ffs((int)hit) - 1;
+          clear = clear && __all_sync(0xffffffffu, lane + 32 * q >= M ||
+                                                       fabsf(pre[q] - near_t) > margin);
+        }
+      }
+      if (clear && found >= 0) return found;
       const R target = P::u(w, 1) * tree_sum(vl, lane, M);
       R acc = R(0);
       int pk = -1, last = -1;
       for (int j = 0; j < M; ++j) {
         const R vj = v[j];
-        if (vj > R(0)) last = j;
+        if (P::positive(vj)) last = j;
         acc = acc + vj;
-        if (target < acc) {
+        if (P::lt(target, acc)) {
           pk = j;
           break;
         }
@@ -229,6 +311,10 @@ struct WarpTraj {
       }
       return __shfl_sync(0xffffffffu, pk, src);
     }
+  }
+
+  __device__ static __forceinline__ float near32(double d) {
+    return ThreadTraj<1, 1, P>::f32_near(d);
   }
 
   // Fast precision: one FP32 inclusive scan of the lanes' sums of their (at most kRPL)
@@ -299,23 +385,27 @@ struct WarpTraj {
       const int s = lane + 32 * q;
       c[q] = 0.0;
       if (s < N) {
-        double acc = (double)sl.x[s];
+        const double xs = f64_of_count(sl.x[s]);
+        double acc = xs;
         for (int e = md.sp_ptr[s]; e < md.sp_ptr[s + 1]; ++e) {
           const int j = md.sp_j[e];
           if (bit(nc, j))
-            acc = acc + (double)md.sp_nu[e] * ((double)sl.K[j] - (double)a[j] * tau);
+            acc = acc + nu_times(md.sp_nu[e], f64_of_count(sl.K[j]) - (double)a[j] * tau);
         }
         c[q] = acc;
-        sl.y[s] = (double)sl.x[s];
+        sl.y[s] = xs;
       }
     }
     __syncwarp();
     for (int it = 0; it < maxit; ++it) {
+      // the propensities at y; critical reactions' are zero in the sums (a zero leaves them)
 #pragma unroll
       for (int q = 0; q < kRPL; ++q) {
         const int j = lane + 32 * q;
-        if (j < M) sl.ay[j] = (double)th[q] * g_real(md, j, sl.y, -1, 0.0);
+        if (j < M)
+          sl.ay[j] = own(nc, q, lane) ? (double)th[q] * g_real(md, j, sl.y, -1, 0.0) : 0.0;
       }
+      for (int e = lane; e < N * N; e += 32) Jm[e] = L(0);
       __syncwarp();
       // right-hand side and Jacobian entries
 #pragma unroll
@@ -323,10 +413,8 @@ struct WarpTraj {
         const int s = lane + 32 * q;
         if (s < N) {
           double acc = 0.0;
-          for (int e = md.sp_ptr[s]; e < md.sp_ptr[s + 1]; ++e) {
-            const int j = md.sp_j[e];
-            if (bit(nc, j)) acc = acc + (double)md.sp_nu[e] * sl.ay[j];
-          }
+          for (int e = md.sp_ptr[s]; e < md.sp_ptr[s + 1]; ++e)
+            acc = acc + nu_times(md.sp_nu[e], sl.ay[md.sp_j[e]]);
           bv[s] = (L)(-((sl.y[s] - c[q]) - tau * acc));
         }
       }
@@ -337,7 +425,7 @@ struct WarpTraj {
           const int nr = md.nreact[j];
           for (int k = 0; k < 3; ++k) {
             L dv = L(0);
-            if (k < nr && bit(nc, j)) {
+            if (k < nr && own(nc, q, lane)) {
               if (analytic) {
                 L v = L(1);
                 for (int kk = 0; kk < nr; ++kk) {
@@ -361,34 +449,49 @@ struct WarpTraj {
         }
       }
       __syncwarp();
-      // Jacobian rows: J[s][q] = [s == q] - tau sum_j nu_js D_jq (j increasing)
+      // Jacobian rows: J[s][q] = [s == q] - tau sum_j nu_js D_jq (j increasing); only the
+      // entries some reaction touches are computed, the others are those of the identity
 #pragma unroll
       for (int q = 0; q < kSPL; ++q) {
         const int s = lane + 32 * q;
         if (s < N) {
           L* row = Jm + (size_t)s * N;
-          for (int cc = 0; cc < N; ++cc) row[cc] = L(0);
+          unsigned long long touched = 0;
           for (int e = md.sp_ptr[s]; e < md.sp_ptr[s + 1]; ++e) {
             const int j = md.sp_j[e];
-            if (!bit(nc, j)) continue;
-            const L v = (L)md.sp_nu[e];
+            const L v = nu_as(md.sp_nu[e], L(0));
             const int nr = md.nreact[j];
             for (int k = 0; k < nr; ++k) {
               const int qq = md.rsp[j][k];
               row[qq] = row[qq] + v * Dm[j * 3 + k];
+              touched |= 1ULL << qq;
             }
           }
-          for (int cc = 0; cc < N; ++cc) row[cc] = (s == cc ? L(1) : L(0)) - taur * row[cc];
+          if (!((touched >> s) & 1ULL)) row[s] = L(1);
+          while (touched != 0) {
+            const int cc = __ffsll((long long)touched) - 1;
+            touched &= touched - 1;
+            row[cc] = (s == cc ? L(1) : L(0)) - taur * row[cc];
+          }
         }
       }
       __syncwarp();
-      // Gaussian elimination with partial pivoting (largest |pivot|, lowest row on ties)
+      // Gaussian elimination with partial pivoting (largest |pivot|, lowest row on ties).
+      // The matrix is sparse (a row has the species that its reactions read), so a column
+      // has a few rows to eliminate: they are found by ballot, their factors are divided in
+      // one step, and each row's update runs over the columns, one per lane (a row whose
+      // factor is zero would be left as it is).  Comparisons are on the integer pipe.  The
+      // dense form, a row per lane, took about 3,400 FP64 instructions for 50 species.
       for (int k = 0; k < N; ++k) {
+        L own_v[kSPL];
         L best = L(-1);
         int piv = N;
-        for (int i = k + lane; i < N; i += 32) {
-          const L v = fabs(Jm[(size_t)i * N + k]);
-          if (v > best) {
+#pragma unroll
+        for (int q = 0; q < kSPL; ++q) {
+          const int i = k + lane + 32 * q;
+          own_v[q] = i < N ? Jm[(size_t)i * N + k] : L(0);
+          const L v = fabs(own_v[q]);
+          if (i < N && pivot_gt(v, best)) {
             best = v;
             piv = i;
           }
@@ -397,12 +500,12 @@ struct WarpTraj {
         for (int d = 16; d >= 1; d >>= 1) {
           const L ob = __shfl_xor_sync(0xffffffffu, best, d);
           const int op = __shfl_xor_sync(0xffffffffu, piv, d);
-          if (ob > best || (ob == best && op < piv)) {
+          if (pivot_gt(ob, best) || (same_bits(ob, best) && op < piv)) {
             best = ob;
             piv = op;
           }
         }
-        if (!(best > L(0)) || piv >= N) return 2;  // zero or non-finite column: singular
+        if (!pivot_gt(best, L(0)) || piv >= N) return 2;  // zero or non-finite column: singular
         if (piv != k) {
           for (int cc = lane; cc < N; cc += 32) {
             const L t = Jm[(size_t)k * N + cc];
@@ -414,23 +517,54 @@ struct WarpTraj {
             bv[k] = bv[piv];
             bv[piv] = t;
           }
+          // row piv now starts with what row k held in this column
+          const L vk = __shfl_sync(0xffffffffu, own_v[0], 0);
+#pragma unroll
+          for (int q = 0; q < kSPL; ++q) {
+            if (k + lane + 32 * q == piv) own_v[q] = vk;
+          }
         }
         __syncwarp();
         const L pk = Jm[(size_t)k * N + k];
         const L bk = bv[k];
-        for (int i = k + 1 + lane; i < N; i += 32) {
-          const L l = Jm[(size_t)i * N + k] / pk;
-          for (int cc = k + 1; cc < N; ++cc)
-            Jm[(size_t)i * N + cc] = Jm[(size_t)i * N + cc] - l * Jm[(size_t)k * N + cc];
-          bv[i] = bv[i] - l * bk;
+#pragma unroll
+        for (int q = 0; q < kSPL; ++q) {
+          const int i = k + lane + 32 * q;
+          const bool on = i > k && i < N && !is_zero(own_v[q]);
+          unsigned rows = __ballot_sync(0xffffffffu, on);
+          if (rows == 0) continue;
+          const L l = on ? own_v[q] / pk : L(0);
+          if (on) bv[i] = bv[i] - l * bk;
+          while (rows != 0) {
+            const int r = __ffs((int)rows) - 1;
+            rows &= rows - 1;
+            const L lr = __shfl_sync(0xffffffffu, l, r);
+            L* row = Jm + (size_t)(k + r + 32 * q) * N;
+            for (int cc = k + 1 + lane; cc < N; cc += 32)
+              row[cc] = row[cc] - lr * Jm[(size_t)k * N + cc];
+          }
         }
         __syncwarp();
       }
-      // column-oriented back substitution
+      // column-oriented back substitution; the divisions by the diagonal share their
+      // reciprocals, taken for all rows at once
+      L inv[kSPL], dia[kSPL];
+#pragma unroll
+      for (int q = 0; q < kSPL; ++q) {
+        const int i = lane + 32 * q;
+        dia[q] = i < N ? Jm[(size_t)i * N + i] : L(1);
+        inv[q] = L(1) / dia[q];
+      }
       for (int i = N - 1; i >= 0; --i) {
-        const L di = bv[i] / Jm[(size_t)i * N + i];
+        const int src = i & 31;
+        const L inv_i = __shfl_sync(0xffffffffu, i < 32 ? inv[0] : inv[kSPL - 1], src);
+        const L dia_i = __shfl_sync(0xffffffffu, i < 32 ? dia[0] : dia[kSPL - 1], src);
+        const L di = div_by_known(bv[i], dia_i, inv_i);
         __syncwarp();
-        for (int rr = lane; rr < i; rr += 32) bv[rr] = bv[rr] - Jm[(size_t)rr * N + i] * di;
+        for (int rr = lane; rr < i; rr += 32) {
+          const L jv = Jm[(size_t)rr * N + i];
+          if (!is_zero(jv)) bv[rr] = bv[rr] - jv * di;
+        }
         if (lane == 0) bv[i] = di;
         __syncwarp();
       }
@@ -469,6 +603,7 @@ struct WarpTraj {
     const uint32_t Mr = (uint32_t)M;
     R* a_s = static_cast<R*>(sl.a);
     R* ac_s = static_cast<R*>(sl.ac);
+    R* scratch = reinterpret_cast<R*>(sl.ay);  // free outside the implicit solve
     uint32_t status = 0;
 
     R th[kRPL];
@@ -501,7 +636,7 @@ struct WarpTraj {
     }
     bad = __any_sync(0xffffffffu, bad);
     __syncwarp();
-    const double T = A.T_per ? A.T[i] : A.T[0];
+    double T = A.T_per ? A.T[i] : A.T[0];
     long long r[kRPL];
     double G[kRPL];
     R g[kRPL], a[kRPL];
@@ -518,7 +653,10 @@ struct WarpTraj {
       status |= ML_ST_BAD_INPUT;
       t = T;
     }
-    if (T != T) t = 0.0;
+    if (T != T) {  // NaN horizon: finishes at once
+      t = 0.0;
+      T = -1.0;
+    }
 
     // Time-grid output: X(t_k) of the right-continuous path; each lane writes its own
     // species, the grid index is warp-uniform.
@@ -553,7 +691,7 @@ struct WarpTraj {
         a[q] = R(0);
         if (j < M) {
           g[q] = g_int(md, j, sl.x);
-          a[q] = th[q] * g[q];
+          a[q] = P::mul(th[q], g[q]);
           a_s[j] = a[q];
         }
       }
@@ -569,7 +707,7 @@ struct WarpTraj {
         const int j = lane + 32 * q;
         if (j < M && (md.rmask[j] & changed) != 0ULL) {
           g[q] = g_int(md, j, sl.x);
-          a[q] = th[q] * g[q];
+          a[q] = P::mul(th[q], g[q]);
           a_s[j] = a[q];
         }
       }
@@ -584,7 +722,7 @@ struct WarpTraj {
     auto ssa_burst_fast = [&](int n_max, R a0_unused) {
       (void)a0_unused;
       const double rem = T - t;
-      const float remf = (float)rem;
+      const float remf = f32_of_f64(rem);
       float el = 0.f, elc = 0.f;
       float Gs[kRPL], Gc[kRPL];
 #pragma unroll
@@ -595,11 +733,18 @@ struct WarpTraj {
 #pragma unroll
       for (int q = 0; q < kSPL; ++q) {
         const int s = lane + 32 * q;
-        if (s < N) xf[s] = (float)sl.x[s];
+        if (s < N) xf[s] = f32_of_count(sl.x[s]);
       }
       __syncwarp();
-      Words4 w = philox_block(k0, k1, id, step, Mr + 2u, 0u);
+      // the random blocks and waiting times' logarithms of the next 32 firings, one per lane
+      Words4 wl{0u, 0u, 0u, 0u};
+      float wait_l = 0.f;
       for (int b = 0; b < n_max; ++b) {
+        if ((b & 31) == 0) {
+          wl = philox_block(k0, k1, id, step, Mr + 2u, (uint32_t)(b + lane));
+          wait_l = -P::log(P::u(wl, 0));
+        }
+        const float wait = __shfl_sync(0xffffffffu, wait_l, b & 31);
         if (b > 0) {  // reactions with a reactant the last firing changed
           const uint64_t changed = fired >= 0 ? md.cmask[fired] : ~0ULL;
 #pragma unroll
@@ -607,7 +752,7 @@ struct WarpTraj {
             const int j = lane + 32 * q;
             if (j < M && (md.rmask[j] & changed) != 0ULL) {
               g[q] = (R)WarpTraj<P>::g_flt(md, j, xf);
-              a[q] = th[q] * g[q];
+              a[q] = P::mul(th[q], g[q]);
             }
           }
         }
@@ -617,14 +762,15 @@ struct WarpTraj {
           to_horizon = true;
           break;
         }
-        const Words4 w_next = philox_block(k0, k1, id, step, Mr + 2u, (uint32_t)b + 1u);
-        const float dt = __fdividef(-P::log(P::u(w, 0)), a0);  // about 2 ulp
+        const Words4 w{0u, 0u, __shfl_sync(0xffffffffu, wl.w2, b & 31),
+                       __shfl_sync(0xffffffffu, wl.w3, b & 31)};
+        const float dt = __fdividef(wait, a0);  // about 2 ulp
         if ((el - elc) + dt > remf) {
           to_horizon = true;
           break;
         }
 #pragma unroll
-        for (int q = 0; q < kRPL; ++q) kahan_add(Gs[q], Gc[q], (float)g[q] * dt);
+        for (int q = 0; q < kRPL; ++q) kahan_fma(Gs[q], Gc[q], (float)g[q], dt);
         kahan_add(el, elc, dt);
         if (kGrid && A.K_obs > 0) {
           record(t + ((double)el - (double)elc), false);  // before the firing: old state
@@ -646,13 +792,12 @@ struct WarpTraj {
         }
         __syncwarp();
         if (kGrid && A.K_obs > 0) record(t + ((double)el - (double)elc), true);
-        w = w_next;
       }
       // the propensities in shared memory (read by the next evaluation's step sizes) are
       // recomputed there; g and a stay current for the horizon term below
-      const double elapsed = (double)el - (double)elc;
+      const double elapsed = f64_of_f32(el) - f64_of_f32(elc);
 #pragma unroll
-      for (int q = 0; q < kRPL; ++q) G[q] = G[q] + ((double)Gs[q] - (double)Gc[q]);
+      for (int q = 0; q < kRPL; ++q) G[q] = G[q] + (f64_of_f32(Gs[q]) - f64_of_f32(Gc[q]));
       if (to_horizon) {
         const double left = rem - elapsed > 0.0 ? rem - elapsed : 0.0;
 #pragma unroll
@@ -669,23 +814,30 @@ struct WarpTraj {
         return;
       }
       int fired = -1;
+      // the random blocks and waiting times' logarithms of the next 32 firings, one per lane
+      Words4 wl{0u, 0u, 0u, 0u};
+      R wait_l = R(0);
       for (int b = 0; b < n_max; ++b) {
+        if ((b & 31) == 0) {
+          wl = philox_block(k0, k1, id, step, Mr + 2u, (uint32_t)(b + lane));
+          wait_l = -P::log(P::u(wl, 0));
+        }
         if (b > 0) {
           update_props(fired);
           a0 = tree_sum(a, lane, M);
         }
-        if (a0 == R(0)) {
+        if (P::zero(a0)) {
           const double rem = T - t;
 #pragma unroll
           for (int q = 0; q < kRPL; ++q) G[q] = G[q] + (double)g[q] * rem;
           t = T;
           return;
         }
-        const Words4 w = philox_block(k0, k1, id, step, Mr + 2u, (uint32_t)b);
-        const R u1 = P::u(w, 0);
-        const R dt = -P::log(u1) / a0;
+        const Words4 w{0u, 0u, __shfl_sync(0xffffffffu, wl.w2, b & 31),
+                       __shfl_sync(0xffffffffu, wl.w3, b & 31)};
+        const R dt = __shfl_sync(0xffffffffu, wait_l, b & 31) / a0;
         const double tn = t + (double)dt;
-        if (tn > T) {
+        if (f64_lt_nn(T, tn)) {
           const double rem = T - t;
 #pragma unroll
           for (int q = 0; q < kRPL; ++q) G[q] = G[q] + (double)g[q] * rem;
@@ -694,8 +846,7 @@ struct WarpTraj {
         }
 #pragma unroll
         for (int q = 0; q < kRPL; ++q) {
-          if (P::kRef) G[q] = G[q] + (double)g[q] * (double)dt;
-          else G[q] = G[q] + (double)(g[q] * dt);  // FP32 increment, FP64 accumulation
+          if (32 * q < M) G[q] = G[q] + (double)g[q] * (double)dt;
         }
         if (kGrid && A.K_obs > 0) {
           record(tn, false);  // points before the firing see the old state
@@ -717,9 +868,9 @@ struct WarpTraj {
       }
     };
 
-    const R eps = (R)A.eps;
+    const R eps = P::eps(A);
     for (;;) {
-      if (!(t < T)) break;
+      if (!f64_lt_nn(t, T)) break;
       if ((long long)step >= A.max_steps) {
         status |= ML_ST_STEP_LIMIT;
         break;
@@ -740,7 +891,7 @@ struct WarpTraj {
       }
       eval_props();
       const R a0 = tree_sum(a, lane, M);
-      if (a0 == R(0)) {
+      if (P::zero(a0)) {
         const double rem = T - t;
 #pragma unroll
         for (int q = 0; q < kRPL; ++q) G[q] = G[q] + (double)g[q] * rem;
@@ -757,7 +908,7 @@ struct WarpTraj {
         for (int q = 0; q < kRPL; ++q) {
           const int j = lane + 32 * q;
           bool crit = false;
-          if (j < M && a[q] > R(0)) {
+          if (j < M && P::positive(a[q])) {
             // min over consumed species of floor(x_s/|nu_js|) below n_c, i.e. some
             // consumed species has x_s < n_c |nu_js|
             for (int e = md.rx_ptr[j]; e < md.rx_ptr[j + 1]; ++e) {
@@ -771,7 +922,7 @@ struct WarpTraj {
         }
         __syncwarp();
         const R a0c = tree_sum(ac, lane, M);
-        const R tau_ex = tau_select(md, a_s, sl.x, nc, eps, lane);
+        const R tau_ex = tau_select(md, a, scratch, sl.x, nc, eps, lane);
         bool implicit = false;
         R tau1 = tau_ex;
         if (A.mode == ML_MODE_ADAPTIVE && md.n_pairs > 0) {
@@ -782,22 +933,12 @@ struct WarpTraj {
             const int j = lane + 32 * q;
             bool on = false;
             if (j < M) {
-              int k = md.partner[j];
-              int lo_j = j, hi_j = k;
-              if (k < 0) {
-                // j may be the higher reaction of a pair: find it
-                for (int jj = 0; jj < j; ++jj)
-                  if (md.partner[jj] == j) {
-                    lo_j = jj;
-                    hi_j = j;
-                    k = jj;
-                    break;
-                  }
-              }
+              const int k = md.pair[j];
+              const int lo_j = k < j ? k : j, hi_j = k < j ? j : k;
               if (k >= 0 && bit(nc, lo_j) && bit(nc, hi_j)) {
                 const R aj = a_s[lo_j], ak = a_s[hi_j];
-                const R lo = aj < ak ? aj : ak;
-                on = fabs(aj - ak) <= (R)A.pe_delta * lo;
+                const R lo = P::lt(aj, ak) ? aj : ak;
+                on = !P::lt(P::mul(P::pe_delta(A), lo), fabs(aj - ak));
               }
             }
             pe[q] = __ballot_sync(0xffffffffu, on);
@@ -807,8 +948,8 @@ struct WarpTraj {
             uint32_t use[kRPL];
 #pragma unroll
             for (int q = 0; q < kRPL; ++q) use[q] = nc[q] & ~pe[q];
-            const R tau_im = tau_select(md, a_s, sl.x, use, eps, lane);
-            if (tau_im > (R)A.stiff_ratio * tau_ex) {
+            const R tau_im = tau_select(md, a, scratch, sl.x, use, eps, lane);
+            if (P::lt(P::mul(P::stiff_ratio(A), tau_ex), tau_im)) {
               implicit = true;
               tau1 = tau_im;
             }
@@ -822,31 +963,32 @@ struct WarpTraj {
             break;
           }
           R tau2 = P::inf();
-          if (a0c > R(0)) {
+          if (P::positive(a0c)) {
             const Words4 w = philox_block(k0, k1, id, step, Mr, 0u);
             tau2 = -P::log(P::u(w, 0)) / a0c;
           }
-          const R tmin = tau1 < tau2 ? tau1 : tau2;
-          if (tmin < (R)A.ssa_factor / a0) {
+          const R tmin = P::lt(tau1, tau2) ? tau1 : tau2;
+          if (P::lt(tmin, P::ssa_factor(A) / a0)) {
             burst = implicit ? A.n_ssa_im : A.n_ssa_ex;
             break;
           }
           const double stop = kGrid ? stop_time() : T;
           const double rem = stop - t;
           R tau = tau1;
-          if (tau2 < tau) tau = tau2;
+          if (P::lt(tau2, tau)) tau = tau2;
           bool at_horizon = false;
-          if ((R)rem <= tau) {
-            tau = (R)rem;
+          const R rmr = P::of_f64(rem);
+          if (!P::lt(tau, rmr)) {
+            tau = rmr;
             at_horizon = true;
           }
-          const bool crit_fire = (tau2 <= tau1) && (tau2 <= (R)rem);
+          const bool crit_fire = !P::lt(tau1, tau2) && !P::lt(rmr, tau2);
           {
             bool over = false;
 #pragma unroll
             for (int q = 0; q < kRPL; ++q) {
               const int j = lane + 32 * q;
-              over = over || (j < M && bit(nc, j) && a[q] * tau > (R)kLeapLimit);
+              over = over || (j < M && own(nc, q, lane) && P::lt((R)kLeapLimit, P::mul(a[q], tau)));
             }
             overflow = __any_sync(0xffffffffu, over);
             if (overflow) break;
@@ -856,15 +998,15 @@ struct WarpTraj {
             const Words4 w = philox_block(k0, k1, id, step, Mr + 1u, 0u);
             cpk = pick(ac_s, ac, Words4{0u, 0u, w.w0, w.w1}, M, lane);
           }
-          const bool implicit_step = implicit && tau > tau_ex;
+          const bool implicit_step = implicit && P::lt(tau_ex, tau);
           long long K[kRPL];
 #pragma unroll
           for (int q = 0; q < kRPL; ++q) {
             const int j = lane + 32 * q;
             K[q] = 0;
             if (j < M) {
-              if (bit(nc, j))
-                K[q] = poisson_draw<P>(a[q] * tau, k0, k1, id, step, (uint32_t)j, status);
+              if (own(nc, q, lane))
+                K[q] = poisson_draw<P>(P::mul(a[q], tau), k0, k1, id, step, (uint32_t)j, status);
               sl.K[j] = K[q];
             }
           }
@@ -889,9 +1031,9 @@ struct WarpTraj {
 #pragma unroll
             for (int q = 0; q < kRPL; ++q) {
               const int j = lane + 32 * q;
-              if (j < M && bit(nc, j)) {
+              if (j < M && own(nc, q, lane)) {
                 const double ayj = (double)th[q] * g_real(md, j, sl.y, -1, 0.0);
-                const double v = (ayj * taud + (double)K[q]) - (double)a[q] * taud;
+                const double v = (ayj * taud + f64_of_count(K[q])) - (double)a[q] * taud;
                 const double rv = round(v);
                 K[q] = !(rv < 0x1p62) ? kCountLimit : (rv > 0.0 ? (long long)rv : 0);
               }
@@ -900,7 +1042,7 @@ struct WarpTraj {
 #pragma unroll
             for (int q = 0; q < kRPL; ++q) {
               const int j = lane + 32 * q;
-              over = over || (j < M && bit(nc, j) && K[q] > kLeapLimitInt);
+              over = over || (j < M && own(nc, q, lane) && K[q] > kLeapLimitInt);
             }
             overflow = __any_sync(0xffffffffu, over);
             if (overflow) break;
@@ -909,7 +1051,7 @@ struct WarpTraj {
           for (int q = 0; q < kRPL; ++q) {
             const int j = lane + 32 * q;
             if (j == cpk) K[q] = 1;
-            else if (j < M && !bit(nc, j)) K[q] = 0;
+            else if (j < M && !own(nc, q, lane)) K[q] = 0;
             if (j < M) sl.K[j] = K[q];
           }
           __syncwarp();
@@ -934,7 +1076,6 @@ struct WarpTraj {
             cnt[3] += 1;
             continue;
           }
-          const double half = (double)tau * 0.5;
           const R half_r = tau * R(0.5);
 #pragma unroll
           for (int q = 0; q < kRPL; ++q) {
@@ -942,8 +1083,8 @@ struct WarpTraj {
             if (j < M) {
               const R gn = g_int(md, j, sl.xn);
               r[q] += K[q];
-              if (P::kRef) G[q] = G[q] + half * ((double)g[q] + (double)gn);
-              else G[q] = G[q] + (double)(half_r * (g[q] + gn));  // FP32 increment
+              // fast precision: an FP32 increment
+              G[q] = G[q] + P::to_f64(half_r * (g[q] + gn));
             }
           }
           __syncwarp();
@@ -953,7 +1094,7 @@ struct WarpTraj {
             if (s < N) sl.x[s] = sl.xn[s];
           }
           __syncwarp();
-          t = at_horizon ? stop : t + (double)tau;
+          t = at_horizon ? stop : t + P::to_f64(tau);
           if (kGrid && A.K_obs > 0) record(t, true);
           cnt[implicit_step ? 1 : 0] += 1;
           step++;
