@@ -198,8 +198,7 @@ std::vector<uint8_t> warp_tables(const ml_model& m) {
     for (int j = 0; j < m.M; ++j) {
       const int v = m.nu[j * m.N + s];
       if (v != 0) {
-        w.sp_j[k] = (int16_t)j;
-        w.sp_nu[k] = (int8_t)v;
+        w.sp_e[k] = (int16_t)(j | (v << 8));
         ++k;
       }
     }

@@ -95,8 +95,7 @@ struct alignas(16) WarpModel {
   // entries (filled up to nnz): per-reaction lists then per-species lists
   int8_t rx_s[kWarpMaxM * 8];
   int8_t rx_nu[kWarpMaxM * 8];
-  int16_t sp_j[kWarpMaxM * 8];
-  int8_t sp_nu[kWarpMaxM * 8];
+  int16_t sp_e[kWarpMaxM * 8];  // reaction (low byte) and net change (high byte, signed)
 };
 
 // Everything a simulation kernel needs besides the model tables.

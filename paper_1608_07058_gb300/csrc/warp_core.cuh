@@ -187,8 +187,8 @@ struct WarpTraj {
       if (s < md.N && md.isreact[s]) {
         R mu = R(0), var = R(0);
         for (int e = md.sp_ptr[s]; e < md.sp_ptr[s + 1]; ++e) {
-          const R aj = am[md.sp_j[e]];
-          const int v = md.sp_nu[e];
+          const int ent = md.sp_e[e], v = ent >> 8;
+          const R aj = am[ent & 0xff];
           if (P::kRef && (v == 1 || v == -1)) {  // the products are exact
             mu = v > 0 ? mu + aj : mu - aj;
             var = var + aj;
@@ -388,9 +388,9 @@ struct WarpTraj {
         const double xs = f64_of_count(sl.x[s]);
         double acc = xs;
         for (int e = md.sp_ptr[s]; e < md.sp_ptr[s + 1]; ++e) {
-          const int j = md.sp_j[e];
+          const int ent = md.sp_e[e], j = ent & 0xff;
           if (bit(nc, j))
-            acc = acc + nu_times(md.sp_nu[e], f64_of_count(sl.K[j]) - (double)a[j] * tau);
+            acc = acc + nu_times(ent >> 8, f64_of_count(sl.K[j]) - (double)a[j] * tau);
         }
         c[q] = acc;
         sl.y[s] = xs;
@@ -414,7 +414,7 @@ struct WarpTraj {
         if (s < N) {
           double acc = 0.0;
           for (int e = md.sp_ptr[s]; e < md.sp_ptr[s + 1]; ++e)
-            acc = acc + nu_times(md.sp_nu[e], sl.ay[md.sp_j[e]]);
+            acc = acc + nu_times(md.sp_e[e] >> 8, sl.ay[md.sp_e[e] & 0xff]);
           bv[s] = (L)(-((sl.y[s] - c[q]) - tau * acc));
         }
       }
@@ -458,8 +458,8 @@ struct WarpTraj {
           L* row = Jm + (size_t)s * N;
           unsigned long long touched = 0;
           for (int e = md.sp_ptr[s]; e < md.sp_ptr[s + 1]; ++e) {
-            const int j = md.sp_j[e];
-            const L v = nu_as(md.sp_nu[e], L(0));
+            const int ent = md.sp_e[e], j = ent & 0xff;
+            const L v = nu_as(ent >> 8, L(0));
             const int nr = md.nreact[j];
             for (int k = 0; k < nr; ++k) {
               const int qq = md.rsp[j][k];
@@ -683,7 +683,75 @@ struct WarpTraj {
     };
     if (kGrid && A.K_obs > 0) record(t, true);
 
+    // Fast precision, networks of order two at most: each own reaction's reactants as offsets
+    // into the FP32 state copy (kept in the leap's xn storage, free between leaps, its entry N
+    // holding 1 for an absent reactant) and the counts below which it is critical, in
+    // registers.  A propensity is then two loads and two or three products without a branch;
+    // the loop over the reactant lists, divergent in their lengths, took about 60
+    // instructions for each of a lane's four reactions, and every SSA firing runs it.
+    float* xf = reinterpret_cast<float*>(sl.xn);
+    int q0[kRPL], q1[kRPL];
+    float need0[kRPL], need1[kRPL];
+    bool quick = !P::kRef && A.n_c <= 100000;
+    if (!P::kRef) {
+#pragma unroll
+      for (int q = 0; q < kRPL; ++q) {
+        const int j = lane + 32 * q;
+        q0[q] = q1[q] = N;
+        need0[q] = need1[q] = 0.f;
+        if (j < M) {
+          const int nr = md.nreact[j];
+          if (nr > 0) q0[q] = md.rsp[j][0];
+          if (nr > 1) q1[q] = md.rsp[j][1];
+          if (nr == 1 && md.rmul[j][0] == 2) q1[q] = -1;  // C(x, 2)
+          int order = 0;
+          for (int k = 0; k < nr; ++k) order += md.rmul[j][k];
+          if (order > 2) quick = false;
+          for (int e = md.rx_ptr[j]; e < md.rx_ptr[j + 1]; ++e) {
+            const int v = md.rx_nu[e];
+            if (v < 0) {  // a consumed species is a reactant
+              const float need = (float)(A.n_c * -v);
+              if (md.rx_s[e] == q0[q]) need0[q] = need;
+              else need1[q] = need;
+            }
+          }
+        }
+      }
+    }
+    quick = __all_sync(0xffffffffu, quick);
+    auto load_xf = [&]() {
+#pragma unroll
+      for (int q = 0; q < kSPL; ++q) {
+        const int s = lane + 32 * q;
+        if (s < N) xf[s] = f32_of_count(sl.x[s]);
+      }
+      if (lane == 0) xf[N] = 1.f;
+      __syncwarp();
+    };
+    // g of the lane's q-th reaction from xf; x: its first reactant's count, y: the second's
+    auto g_quick = [&](int q, float& x, float& y) {
+      x = xf[q0[q]];
+      y = xf[q1[q] < 0 ? N : q1[q]];
+      const float pair = x < 2.f ? 0.f : (x * (x - 1.f)) * 0.5f;
+      return q1[q] < 0 ? pair : x * y;
+    };
+
     auto eval_props = [&]() {
+      if constexpr (!P::kRef) {
+        if (quick) {
+          load_xf();
+#pragma unroll
+          for (int q = 0; q < kRPL; ++q) {
+            const int j = lane + 32 * q;
+            float x, y;
+            g[q] = j < M ? (R)g_quick(q, x, y) : R(0);
+            a[q] = P::mul(th[q], g[q]);
+            if (j < M) a_s[j] = a[q];
+          }
+          __syncwarp();
+          return;
+        }
+      }
 #pragma unroll
       for (int q = 0; q < kRPL; ++q) {
         const int j = lane + 32 * q;
@@ -729,13 +797,7 @@ struct WarpTraj {
       for (int q = 0; q < kRPL; ++q) Gs[q] = Gc[q] = 0.f;
       bool to_horizon = false;
       int fired = -1;
-      float* xf = reinterpret_cast<float*>(sl.xn);
-#pragma unroll
-      for (int q = 0; q < kSPL; ++q) {
-        const int s = lane + 32 * q;
-        if (s < N) xf[s] = f32_of_count(sl.x[s]);
-      }
-      __syncwarp();
+      load_xf();
       // the random blocks and waiting times' logarithms of the next 32 firings, one per lane
       Words4 wl{0u, 0u, 0u, 0u};
       float wait_l = 0.f;
@@ -745,7 +807,16 @@ struct WarpTraj {
           wait_l = -P::log(P::u(wl, 0));
         }
         const float wait = __shfl_sync(0xffffffffu, wait_l, b & 31);
-        if (b > 0) {  // reactions with a reactant the last firing changed
+        if (b > 0 && quick) {
+#pragma unroll
+          for (int q = 0; q < kRPL; ++q) {
+            if (32 * q < M) {
+              float x, y;
+              g[q] = lane + 32 * q < M ? (R)g_quick(q, x, y) : R(0);
+              a[q] = P::mul(th[q], g[q]);
+            }
+          }
+        } else if (b > 0) {  // reactions with a reactant the last firing changed
           const uint64_t changed = fired >= 0 ? md.cmask[fired] : ~0ULL;
 #pragma unroll
           for (int q = 0; q < kRPL; ++q) {
@@ -908,7 +979,15 @@ struct WarpTraj {
         for (int q = 0; q < kRPL; ++q) {
           const int j = lane + 32 * q;
           bool crit = false;
-          if (j < M && P::positive(a[q])) {
+          if (quick) {
+            if constexpr (!P::kRef) {
+              float x, y;
+              if (j < M) {
+                g_quick(q, x, y);
+                crit = a[q] > R(0) && (x < need0[q] || y < need1[q]);
+              }
+            }
+          } else if (j < M && P::positive(a[q])) {
             // min over consumed species of floor(x_s/|nu_js|) below n_c, i.e. some
             // consumed species has x_s < n_c |nu_js|
             for (int e = md.rx_ptr[j]; e < md.rx_ptr[j + 1]; ++e) {
@@ -1062,7 +1141,7 @@ struct WarpTraj {
             if (s < N) {
               long long v = sl.x[s];
               for (int e = md.sp_ptr[s]; e < md.sp_ptr[s + 1]; ++e)
-                v += (long long)md.sp_nu[e] * sl.K[md.sp_j[e]];
+                v += (long long)(md.sp_e[e] >> 8) * sl.K[md.sp_e[e] & 0xff];
               sl.xn[s] = v;
               if (v < 0) negative = true;
             }
