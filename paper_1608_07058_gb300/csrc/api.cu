@@ -47,6 +47,7 @@ int cuda_fail(cudaError_t e, const char* where) {
 // (two measured 10 % slower on 10,007 reference-precision gene-expression trajectories and
 // on 10,000 dimerisation trajectories with a time grid: they share the FP64 unit).
 constexpr int kSpreadWarps = 4;
+constexpr int64_t kRefWarpMax = 0;
 constexpr int kQueueSlots = 256;  // in-flight persistent launches per model and device
 
 struct GraphCache {
@@ -122,6 +123,7 @@ std::vector<uint8_t> build_thread_tables(const ml_model& m) {
         t.rx[j] += (1u << 24) | (((uint32_t)t.ord[j][s] << 4 | (uint32_t)s) << (8 * k));
       }
     }
+    if (j < m.M && m.otot[j] > 2) t.rx[j] |= 0x80000000u;
   }
   for (int j = 0; j < m.M && j < MM; ++j)  // the variant always holds the model (M <= MM)
     if (m.partner[j] > j) t.partner[j] = (int8_t)m.partner[j];
@@ -481,8 +483,9 @@ int make_plan(ml_model* m, DeviceState& st, const ml_sim_params& p, int64_t n_tr
   auto tk = st.tuned.find({p.precision, p.form});
   const Tuned* tuned = tk == st.tuned.end() ? nullptr : &tk->second;
   if (shape == ML_SHAPE_AUTO) {
+    const bool small = p.precision == ML_PREC_REF_FP64 && n_traj <= kRefWarpMax && warp_fits(*m);
     shape = tuned && tuned->shape ? tuned->shape
-                                  : (variant >= 0 ? ML_SHAPE_THREAD : ML_SHAPE_WARP);
+                                  : (variant >= 0 && !small ? ML_SHAPE_THREAD : ML_SHAPE_WARP);
   }
   const int req_shape = shape;
   // a call with time-grid output runs the grid build of the sequential driver (the

@@ -55,7 +55,8 @@ struct alignas(16) ThreadModel {
   double rates[MM];
   float nuf[MM][NM];    // nu_js as FP32 (updates of the fast SSA slice's FP32 state copy)
   // reactants of reaction j in one word, in increasing species: byte k = species of the
-  // k-th (low nibble) and its multiplicity (high nibble), byte 3 = their number (0..3)
+  // k-th (low nibble) and its multiplicity (high nibble), byte 3 = their number (0..3), and
+  // the top bit set when the orders add up to 3
   uint32_t rx[MM];
   int8_t ord[MM][NM];   // m_js
   int8_t nu[MM][NM];    // nu_js

@@ -65,11 +65,17 @@ template <>
 __device__ __forceinline__ double of_count<double>(long long x) { return f64_of_count(x); }
 
 // C(v, m) for m = 1, 2, 3 on a real argument, in this operation order.
+// The third order, with its division, is out of line: the precompiled kernels have a site per
+// reactant, and their code size is what slows them down (instruction fetch).
+template <class R>
+__device__ __noinline__ R comb_three(R v) {
+  return ((v * (v - R(1))) * (v - R(2))) / R(6);
+}
 template <class R>
 __device__ __forceinline__ R comb_factor(R v, int m) {
   if (m == 1) return v;
   if (m == 2) return (v * (v - R(1))) * R(0.5);
-  return ((v * (v - R(1))) * (v - R(2))) / R(6);
+  return comb_three<R>(v);
 }
 
 // C(x, m) of a count: as comb_factor on the converted count.  In FP64 C(x, 2) is an integer
@@ -83,10 +89,14 @@ __device__ __forceinline__ R comb_count(long long x, int m) {
 
 // d/dv C(v, m): 1, v - 1/2, (3 v^2 - 6 v + 2) / 6, in this operation order.
 template <class T>
+__device__ __noinline__ T comb_three_deriv(T v) {
+  return ((T(3) * (v * v) - T(6) * v) + T(2)) / T(6);
+}
+template <class T>
 __device__ __forceinline__ T comb_factor_deriv(T v, int m) {
   if (m == 1) return T(1);
   if (m == 2) return v - T(0.5);
-  return ((T(3) * (v * v) - T(6) * v) + T(2)) / T(6);
+  return comb_three_deriv<T>(v);
 }
 
 // C(x + z, m) - C(x, m) written as z times a polynomial, so that no two large nearby
@@ -157,7 +167,7 @@ __device__ __forceinline__ void kahan_fma(float& s, float& c, float a, float b) 
 
 // Highest-order-reaction factor h_s (Cao 2006) from the species' flags and count.
 template <class R>
-__device__ __forceinline__ R hor_factor(uint8_t f, long long x) {
+__device__ __forceinline__ R hor_factor_at(uint8_t f, long long x) {
   const R xd = of_count<R>(x);
   R h = R(0);
   if (f & kHorO1) h = lt_pos(h, R(1)) ? R(1) : h;
@@ -176,6 +186,17 @@ __device__ __forceinline__ R hor_factor(uint8_t f, long long x) {
     h = lt_pos(h, v) ? v : h;
   }
   return h;
+}
+
+template <class R>
+__device__ __noinline__ R hor_factor_call(uint8_t f, long long x) {
+  return hor_factor_at<R>(f, x);
+}
+// Out of line where the flags are read at run time (four divisions), inline where they are
+// compiled in.
+template <class R, bool kInline = false>
+__device__ __forceinline__ R hor_factor(uint8_t f, long long x) {
+  return kInline ? hor_factor_at<R>(f, x) : hor_factor_call<R>(f, x);
 }
 
 struct PrecRef {
@@ -524,6 +545,11 @@ __device__ __forceinline__ int poisson_invert_at(typename P::R mu, typename P::R
   else return poisson_invert<P>(mu, u);
 }
 
+template <class P>
+__device__ __noinline__ int poisson_invert_call(typename P::R mu, typename P::R u) {
+  return poisson_invert_at<P>(mu, u);
+}
+
 // Poisson(mu) for mu < 10: 0 for mu <= 0 (no draw).
 template <class P>
 __device__ __noinline__ int poisson_small(typename P::R mu, uint32_t k0, uint32_t k1,
@@ -558,8 +584,10 @@ __device__ __forceinline__ bool abs_gt(double a, double b) { return f64_abs_gt(a
 __device__ __forceinline__ bool abs_gt(float a, float b) { return fabsf(a) > fabsf(b); }
 
 // v t for a net change v: the common changes by one are exact without a product.
+__device__ __noinline__ inline double nu_times_call(int v, double t) { return f64_of_i32(v) * t; }
 __device__ __forceinline__ double nu_times(int v, double t) {
-  return v == 1 ? t : v == -1 ? -t : f64_of_i32(v) * t;
+  return v == 1 ? t : v == -1 ? -t : v == 2 || v == -2 ? (v > 0 ? t + t : -(t + t))
+                                                     : nu_times_call(v, t);
 }
 __device__ __forceinline__ float nu_times(int v, float t) { return (float)v * t; }
 
@@ -574,31 +602,66 @@ struct ThreadTraj {
   // product in increasing s, 0 when some x_s < m_js.  The code is a tenth of the loop over
   // all (reaction, species) pairs with a branch per order, which the precompiled kernels
   // ran before: their stalls were instruction fetch.
+  // Orders above two are out of line (bit 31 of the word).
+  template <class V>
+  __device__ static __forceinline__ V sel(const V (&x)[NM], int sp) {
+    V v = x[0];
+#pragma unroll
+    for (int s = 1; s < NM; ++s) v = s == sp ? x[s] : v;
+    return v;
+  }
   template <class V, class F>
-  __device__ static __forceinline__ auto g_word(uint32_t rx, const V (&x)[NM], F comb) {
+  __device__ static __forceinline__ auto g_slots(uint32_t rx, const V (&x)[NM], F comb) {
     using O = decltype(comb(x[0], 1));
     O v = O(1);
     bool zero = false;
-    const int nr = (int)(rx >> 24);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      if (k < nr) {
-        const int sp = (int)(rx >> (8 * k)) & 15, m = (int)(rx >> (8 * k + 4)) & 15;
-        V xs = x[0];
-#pragma unroll
-        for (int s = 1; s < NM; ++s) xs = s == sp ? x[s] : xs;
-        zero = zero || xs < (V)m;
-        const O f = comb(xs, m);
-        v = k == 0 ? f : v * f;
-      }
+    const int nr = (int)(rx >> 24) & 3;
+    for (int k = 0; k < nr; ++k) {
+      const int m = (int)(rx >> (8 * k + 4)) & 15;
+      const V xs = sel(x, (int)(rx >> (8 * k)) & 15);
+      zero = zero || xs < (V)m;
+      const O f = comb(xs, m);
+      v = k == 0 ? f : v * f;
     }
     return zero ? O(0) : v;
+  }
+  __device__ static __noinline__ R g_int_slots(uint32_t rx, const long long (&x)[NM]) {
+    return g_slots(rx, x, [](long long xs, int m) { return comb_count<R>(xs, m); });
+  }
+  __device__ static __noinline__ float g_flt_slots(uint32_t rx, const float (&x)[NM]) {
+    return g_slots(rx, x, [](float xs, int m) { return comb_factor<float>(xs, m); });
+  }
+  // Order two at most: 1, x, C(x, 2) or x y.
+  __device__ static __forceinline__ float g_flt_word(uint32_t rx, const float (&x)[NM]) {
+    const float u = sel(x, (int)rx & 15), v = sel(x, (int)(rx >> 8) & 15);
+    const uint32_t nr = rx >> 24;
+    const float pair = u < 2.f ? 0.f : (u * (u - 1.f)) * 0.5f;
+    const float one = (rx & 0x20u) ? pair : u;
+    return nr == 0u ? 1.f : nr == 1u ? one : u * v;
+  }
+  __device__ static __forceinline__ R g_int_word(uint32_t rx, const long long (&x)[NM]) {
+    const uint32_t nr = rx >> 24;
+    if constexpr (sizeof(R) == 4) {
+      float xf[NM];
+#pragma unroll
+      for (int s = 0; s < NM; ++s) xf[s] = f32_of_count(x[s]);
+      return g_flt_word(rx, xf);
+    } else {
+      if (nr == 0u) return R(1);
+      const long long u = sel(x, (int)rx & 15);
+      if (nr == 1u) {
+        if (rx & 0x20u) return u < 2 ? R(0) : comb_count<R>(u, 2);
+        return of_count<R>(u);
+      }
+      return of_count<R>(u) * of_count<R>(sel(x, (int)(rx >> 8) & 15));
+    }
   }
 
   // g_j at an integer state (0 when some x_s < m_js), product in increasing s.
   __device__ static __forceinline__ R g_int(const Model& md, int j, const long long (&x)[NM]) {
     if constexpr (!Model::kCompiled) {
-      return g_word(md.rx[j], x, [](long long xs, int m) { return comb_count<R>(xs, m); });
+      const uint32_t rx = md.rx[j];
+      return (int)rx < 0 ? g_int_slots(rx, x) : g_int_word(rx, x);
     } else {
       R v = R(1);
       bool zero = false;
@@ -618,7 +681,8 @@ struct ThreadTraj {
   // 2^24, where it equals g_int; above, FP32 rounds the count as g_int's conversion does).
   __device__ static __forceinline__ float g_flt(const Model& md, int j, const float (&xf)[NM]) {
     if constexpr (!Model::kCompiled) {
-      return g_word(md.rx[j], xf, [](float xs, int m) { return comb_factor<float>(xs, m); });
+      const uint32_t rx = md.rx[j];
+      return (int)rx < 0 ? g_flt_slots(rx, xf) : g_flt_word(rx, xf);
     } else {
       float v = 1.f;
       bool zero = false;
@@ -640,15 +704,12 @@ struct ThreadTraj {
     double v = 1.0;
     if constexpr (!Model::kCompiled) {
       const uint32_t rx = md.rx[j];
-      const int nr = (int)(rx >> 24);
+      const int nr = (int)(rx >> 24) & 3;
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
         if (k < nr) {
-          const int sp = (int)(rx >> (8 * k)) & 15, m = (int)(rx >> (8 * k + 4)) & 15;
-          double ys = y[0];
-#pragma unroll
-          for (int s = 1; s < NM; ++s) ys = s == sp ? y[s] : ys;
-          const double f = comb_factor<double>(ys, m);
+          const int m = (int)(rx >> (8 * k + 4)) & 15;
+          const double f = comb_factor<double>(sel(y, (int)(rx >> (8 * k)) & 15), m);
           v = k == 0 ? f : v * f;
         }
       }
@@ -697,6 +758,17 @@ struct ThreadTraj {
   // tau_s = min(bound/|mu|, bound^2/var); the minimum over species.
   __device__ static __forceinline__ R tau_select(const Model& md, const R (&a)[MM],
                                                  const long long (&x)[NM], uint32_t use, R eps) {
+    if constexpr (Model::kCompiled) return tau_select_at(md, a, x, use, eps);
+    else return tau_select_call(md, a, x, use, eps);
+  }
+  __device__ static __noinline__ R tau_select_call(const Model& md, const R (&a)[MM],
+                                                   const long long (&x)[NM], uint32_t use,
+                                                   R eps) {
+    return tau_select_at(md, a, x, use, eps);
+  }
+  __device__ static __forceinline__ R tau_select_at(const Model& md, const R (&a)[MM],
+                                                    const long long (&x)[NM], uint32_t use,
+                                                    R eps) {
     R tau = P::inf();
 #pragma unroll
     for (int s = 0; s < NM; ++s) {
@@ -715,9 +787,9 @@ struct ThreadTraj {
             }
           }
         }
-        const R h = hor_factor<R>(md.hor[s], x[s]);
         R bound = eps * of_count<R>(x[s]);
-        if (md.hor[s] != kHorO1) bound = bound / h;  // h = 1 for a first-order reactant
+        if (md.hor[s] != kHorO1)  // h = 1 for a first-order reactant
+          bound = bound / hor_factor<R, Model::kCompiled>(md.hor[s], x[s]);
         if (P::lt(bound, R(1))) bound = R(1);
         const R t1 = bound / fabs(mu);
         const R t2 = (bound * bound) / var;
@@ -1139,6 +1211,166 @@ struct ImplicitIo {
   float th[MM];
 };
 
+// The implicit leap on tables read at run time: the operations of implicit_solve (kRecip
+// false: the canonical order, a division per Jacobian entry, eliminated row and unknown) or of
+// implicit_leap_wide (true: reciprocals), with loops over the real sizes and arrays in local
+// memory.  The unrolled form carries a branch per (reaction, species, order) and a division
+// sequence per Jacobian entry: the precompiled reference kernel waited 20 cycles for an
+// instruction (20,000 dimerisation trajectories), while a local load is short beside the 64
+// cycles of an FP64 instruction.  Entries that are zero need no elimination.  On success K
+// holds the firing counts.  Returns 0 converged, 1 not converged, 2 singular.
+template <int NM, int MM, class MDL, bool kRecip>
+__device__ __noinline__ int implicit_leap_rolled(const MDL& md, const long long (&x)[NM],
+                                                 long long (&K)[MM], const double (&th)[MM],
+                                                 const double (&ax)[MM], uint32_t nc, double tau,
+                                                 double tol, int maxit, double fd_h,
+                                                 bool analytic) {
+  const int N = md.N, M = md.M;
+  double y[NM], c[NM], ay[MM], yp[NM], he[NM], A[NM][NM], b[NM], inv[NM];
+  auto g_at = [&](uint32_t rx) {
+    double v = 1.0;
+    const int nr = (int)(rx >> 24) & 3;
+#pragma unroll 1
+    for (int k = 0; k < nr; ++k) {
+      const double f = comb_factor<double>(y[(rx >> (8 * k)) & 15], (int)(rx >> (8 * k + 4)) & 15);
+      v = k == 0 ? f : v * f;
+    }
+    return v;
+  };
+#pragma unroll 1
+  for (int s = 0; s < N; ++s) {
+    y[s] = f64_of_count(x[s]);
+    double acc = y[s];
+#pragma unroll 1
+    for (int j = 0; j < M; ++j) {
+      const int v = md.nu[j][s];
+      if (((nc >> j) & 1u) && v != 0) acc = acc + nu_times(v, f64_of_count(K[j]) - ax[j] * tau);
+    }
+    c[s] = acc;
+  }
+  int rc = 1;
+#pragma unroll 1
+  for (int it = 0; it < maxit; ++it) {
+#pragma unroll 1
+    for (int j = 0; j < M; ++j) ay[j] = th[j] * g_at(md.rx[j]);
+#pragma unroll 1
+    for (int s = 0; s < N; ++s) {
+      double acc = 0.0;
+#pragma unroll 1
+      for (int j = 0; j < M; ++j) {
+        const int v = md.nu[j][s];
+        if (((nc >> j) & 1u) && v != 0) acc = acc + nu_times(v, ay[j]);
+      }
+      b[s] = -((y[s] - c[s]) - tau * acc);
+#pragma unroll 1
+      for (int q = 0; q < N; ++q) A[s][q] = 0.0;
+      if (!analytic) {
+        const double h = fd_h * (f64_abs_gt(y[s], 1.0) ? fabs(y[s]) : 1.0);
+        yp[s] = y[s] + h;
+        he[s] = yp[s] - y[s];
+        if (kRecip) he[s] = 1.0 / he[s];
+      }
+    }
+#pragma unroll 1
+    for (int j = 0; j < M; ++j) {
+      const uint32_t rx = md.rx[j];
+      const int nr = ((nc >> j) & 1u) ? (int)(rx >> 24) & 3 : 0;
+#pragma unroll 1
+      for (int k = 0; k < nr; ++k) {
+        const int q = (int)(rx >> (8 * k)) & 15;
+        double D;
+        if (analytic) {
+          double v = 1.0;
+#pragma unroll 1
+          for (int kk = 0; kk < nr; ++kk) {
+            const double yv = y[(rx >> (8 * kk)) & 15];
+            const int m = (int)(rx >> (8 * kk + 4)) & 15;
+            v = v * (kk == k ? comb_factor_deriv<double>(yv, m) : comb_factor<double>(yv, m));
+          }
+          D = th[j] * v;
+        } else {
+          const double keep = y[q];
+          y[q] = yp[q];
+          const double diff = th[j] * g_at(rx) - ay[j];
+          y[q] = keep;
+          D = kRecip ? diff * he[q] : diff / he[q];
+        }
+#pragma unroll 1
+        for (int s = 0; s < N; ++s) {
+          const int v = md.nu[j][s];
+          if (v != 0) A[s][q] = A[s][q] + nu_times(v, D);
+        }
+      }
+    }
+#pragma unroll 1
+    for (int s = 0; s < N; ++s) {
+#pragma unroll 1
+      for (int q = 0; q < N; ++q) {
+        const double e = s == q ? 1.0 : 0.0;
+        A[s][q] = (__double_as_longlong(A[s][q]) << 1) == 0 ? e : e - tau * A[s][q];
+      }
+    }
+#pragma unroll 1
+    for (int k = 0; k < N; ++k) {
+      int piv = k;
+      double best = fabs(A[k][k]);
+#pragma unroll 1
+      for (int i = k + 1; i < N; ++i) {
+        if (f64_abs_gt(A[i][k], best)) {
+          best = fabs(A[i][k]);
+          piv = i;
+        }
+      }
+      if (kRecip ? !f64_abs_gt(best, 0.0) : best == 0.0) return 2;
+      if (piv != k) {
+#pragma unroll 1
+        for (int cc = 0; cc < N; ++cc) {
+          const double t = A[k][cc];
+          A[k][cc] = A[piv][cc];
+          A[piv][cc] = t;
+        }
+        const double t = b[k];
+        b[k] = b[piv];
+        b[piv] = t;
+      }
+      if (kRecip) inv[k] = 1.0 / A[k][k];
+#pragma unroll 1
+      for (int i = k + 1; i < N; ++i) {
+        if ((__double_as_longlong(A[i][k]) << 1) == 0) continue;
+        const double l = kRecip ? A[i][k] * inv[k] : A[i][k] / A[k][k];
+#pragma unroll 1
+        for (int cc = k + 1; cc < N; ++cc) A[i][cc] = A[i][cc] - l * A[k][cc];
+        b[i] = b[i] - l * b[k];
+      }
+    }
+    double dmax = 0.0, ymax = 0.0;
+#pragma unroll 1
+    for (int i = N - 1; i >= 0; --i) {
+      const double d = kRecip ? b[i] * inv[i] : b[i] / A[i][i];
+#pragma unroll 1
+      for (int rr = 0; rr < i; ++rr) b[rr] = b[rr] - A[rr][i] * d;
+      y[i] = y[i] + d;
+      if (f64_abs_gt(d, dmax)) dmax = fabs(d);
+      if (f64_abs_gt(y[i], ymax)) ymax = fabs(y[i]);
+    }
+    if (dmax <= tol * (ymax > 1.0 ? ymax : 1.0)) {
+      rc = 0;
+      break;
+    }
+  }
+  if (rc == 0) {
+#pragma unroll 1
+    for (int j = 0; j < M; ++j) {
+      if ((nc >> j) & 1u) {
+        const double v = (th[j] * g_at(md.rx[j]) * tau + f64_of_count(K[j])) - ax[j] * tau;
+        const double rv = round(v);
+        K[j] = !(rv < 0x1p62) ? kCountLimit : (rv > 0.0 ? (long long)rv : 0);
+      }
+    }
+  }
+  return rc;
+}
+
 // Fast precision, FP64 implicit leap (Rathinam 2003): FP64 propensities a_j(x) =
 // theta_j g_j(x) from the FP32 rate constants, Newton's method from y = x with the FP64
 // residual F(y) = y - c - tau sum_j nu_j a_j(y), Jacobian (forward differences or exact),
@@ -1161,6 +1393,9 @@ __device__ __noinline__ int implicit_leap_wide(const MDL& md,
     th[j] = f64_of_f32(io.th[j]);
     ax[j] = th[j] * TR::g_int(md, j, io.x);
   }
+  if constexpr (!MDL::kCompiled)
+    return implicit_leap_rolled<NM, MM, MDL, true>(md, io.x, io.K, th, ax, nc, tau, tol, maxit,
+                                                   fd_h, analytic);
 #pragma unroll
   for (int s = 0; s < NM; ++s) {
     const double xs = f64_of_count(io.x[s]);
@@ -1950,12 +2185,15 @@ struct ThreadLane {
         Words4 first[MM];
 #pragma unroll
         for (int j = 0; j < MM; ++j)
-          if (MM <= 6 || j < A.M) first[j] = philox_block(k0, k1, id, step, (uint32_t)j, 0u);
+          if (Model::kCompiled || j < A.M)
+            first[j] = philox_block(k0, k1, id, step, (uint32_t)j, 0u);
 #pragma unroll
         for (int j = 0; j < MM; ++j) {
           mus[j] = P::mul(a[j], tau);
           if (((nc >> j) & 1u) && P::positive(mus[j])) {
-            if (P::lt(mus[j], R(10))) K[j] = poisson_invert_at<P>(mus[j], P::u(first[j], 0));
+            if (P::lt(mus[j], R(10)))
+              K[j] = Model::kCompiled ? poisson_invert_at<P>(mus[j], P::u(first[j], 0))
+                                      : poisson_invert_call<P>(mus[j], P::u(first[j], 0));
             else big |= 1u << j;
           }
         }
@@ -1993,7 +2231,11 @@ struct ThreadLane {
           if ((by_trials >> j) & 1u) K[j] = drawn[j];
         if (implicit_step) {
           int rc;
-          if constexpr (P::kRef) {
+          if constexpr (P::kRef && !Model::kCompiled) {
+            rc = implicit_leap_rolled<NM, MM, Model, false>(
+                md, x, K, th, a, nc, tau, A.newton_tol, A.newton_maxit, A.fd_h,
+                A.jacobian == ML_JAC_ANALYTIC);
+          } else if constexpr (P::kRef) {
             double y[NM];
             const double taud = (double)tau;
             rc = TT::implicit_solve(md, th, x, nc, K, a, taud, A.newton_tol, A.newton_maxit,

@@ -116,9 +116,12 @@ struct WarpTraj {
       const int j = lane + 32 * q;
       if (j < M) s = (q == 0) ? v[q] : s + v[q];
     }
+    // a level whose upper lanes are all empty adds zeros: left out (the values are not
+    // negative), and the total is then lane 0's
 #pragma unroll
-    for (int d = 16; d >= 1; d >>= 1) s = s + __shfl_xor_sync(0xffffffffu, s, d);
-    return s;
+    for (int d = 16; d >= 1; d >>= 1)
+      if (M > d) s = s + __shfl_xor_sync(0xffffffffu, s, d);
+    return M > 16 ? s : __shfl_sync(0xffffffffu, s, 0);
   }
 
   __device__ static __forceinline__ R g_int(const WarpModel& md, int j, const long long* x) {
@@ -197,9 +200,9 @@ struct WarpTraj {
             var = P::mad((R)(v * v), aj, var);
           }
         }
-        const R h = hor_factor<R>(md.hor[s], x[s]);
         R bound = eps * of_count<R>(x[s]);
-        if (md.hor[s] != kHorO1) bound = bound / h;  // h = 1 for a first-order reactant
+        if (md.hor[s] != kHorO1)  // h = 1 for a first-order reactant
+          bound = bound / hor_factor<R>(md.hor[s], x[s]);
         if (P::lt(bound, R(1))) bound = R(1);
         const R t1 = bound / fabs(mu);
         const R t2 = (bound * bound) / var;
