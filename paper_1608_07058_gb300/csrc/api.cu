@@ -47,7 +47,6 @@ int cuda_fail(cudaError_t e, const char* where) {
 // (two measured 10 % slower on 10,007 reference-precision gene-expression trajectories and
 // on 10,000 dimerisation trajectories with a time grid: they share the FP64 unit).
 constexpr int kSpreadWarps = 4;
-constexpr int64_t kRefWarpMax = 0;
 constexpr int kQueueSlots = 256;  // in-flight persistent launches per model and device
 
 struct GraphCache {
@@ -395,7 +394,14 @@ int ensure_tables(ml_model* m, DeviceState& st, int shape, int variant) {
       }
       st.thread_tables[variant] = d;
     }
-  } else if (!st.warp_tables) {
+  }
+  // The warp kernel's tables too where the model fits both, and its reference builds loaded:
+  // shape AUTO takes one or the other by the size of the batch, and a call that a program
+  // captures after warming up with another size must not be the one that allocates.
+  if (!st.warp_tables && (shape == ML_SHAPE_WARP || warp_fits(*m))) {
+    cudaFuncAttributes fa;
+    ML_CUDA_TRY(cudaFuncGetAttributes(&fa, warp_entry(ML_PREC_REF_FP64).kernel));
+    ML_CUDA_TRY(cudaFuncGetAttributes(&fa, warp_grid_entry(ML_PREC_REF_FP64).kernel));
     std::vector<uint8_t> b = warp_tables(*m);
     void* d = nullptr;
     ML_CUDA_TRY(cudaMalloc(&d, b.size()));
@@ -475,15 +481,35 @@ struct Plan {
   int per_warp = 32;  // trajectories a warp runs at a time (thread kernels)
 };
 
-// Chooses the kernel and launch shape for one call (model lock held).
+// Reference precision: the largest batch that shape AUTO runs one trajectory per warp, where
+// a trajectory's FP64 operations are spread over the lanes, although the model fits one
+// thread (both kernels give the same bits).  Measured on 152 SMs, thread / warp kernel in ms:
+// equal horizons and rate constants, immigration-death 1,216: 5.8 / 4.3, 2,000: 6.3 / 8.0,
+// dimerisation 1,216: 1.9 / 1.2, 4,000: 3.6 / 4.4 -- up to the warps resident at once (8 per
+// SM); their own horizons and rate constants per trajectory, where the longest ones decide:
+// immigration-death 4,000: 16.9 / 15.5, 8,000: 15.2 / 17.2, dimerisation 4,000: 13.5 / 9.5,
+// 8,000: 15.9 / 16.9, gene expression (6 reactions) 4,000: 386 / 194, 10,007: 527 / 357,
+// 16,000: 580 / 437 -- up to 4 of them per warp, 12 with more than 4 reactions.  Kernels
+// compiled for the model are about 1.5 times as fast: 1 and 4 (gene expression 3,000: 275 / 197).
+int64_t ref_warp_limit(const ml_model& m, const DeviceState& st, const ml_sim_params& p,
+                       bool ragged) {
+  const int64_t resident = (int64_t)st.sm_count * 8;
+  if (!ragged) return resident;
+  const bool large = m.M > 4;
+  return resident * (p.specialize ? (large ? 4 : 1) : (large ? 12 : 4));
+}
+
+// Chooses the kernel and launch shape for one call (model lock held).  ragged: the call gives
+// every trajectory its own rate constants and horizon.
 int make_plan(ml_model* m, DeviceState& st, const ml_sim_params& p, int64_t n_traj,
-              Plan* plan, bool grid_out = false) {
+              Plan* plan, bool ragged, bool grid_out = false) {
   int shape = p.shape;
   const int variant = thread_variant_for(*m);
   auto tk = st.tuned.find({p.precision, p.form});
   const Tuned* tuned = tk == st.tuned.end() ? nullptr : &tk->second;
   if (shape == ML_SHAPE_AUTO) {
-    const bool small = p.precision == ML_PREC_REF_FP64 && n_traj <= kRefWarpMax && warp_fits(*m);
+    const bool small = p.precision == ML_PREC_REF_FP64 && warp_fits(*m) &&
+                       n_traj <= ref_warp_limit(*m, st, p, ragged);
     shape = tuned && tuned->shape ? tuned->shape
                                   : (variant >= 0 && !small ? ML_SHAPE_THREAD : ML_SHAPE_WARP);
   }
@@ -991,7 +1017,7 @@ int ml_simulate_grid(const ml_model* cm, int64_t n_traj, const double* theta,
   rc = device_state(m, &st, &dev);
   if (rc != ML_OK) return rc;
   Plan plan;
-  rc = make_plan(m, *st, p, n_traj, &plan, K > 0 && n_traj > 0);
+  rc = make_plan(m, *st, p, n_traj, &plan, theta && T_per_traj, K > 0 && n_traj > 0);
   if (rc != ML_OK) return rc;
   mlk::SimArgs a;
   fill_args(m, p, n_traj, theta, x0, x0_per_traj, T, T_per_traj, seed, id_base, X, r, G,
@@ -1150,7 +1176,7 @@ int ml_autotune(ml_model* m, int64_t n_traj, const double* theta, const int64_t*
         DeviceState* st = nullptr;
         int dev = 0;
         Plan plan;
-        if (device_state(m, &st, &dev) == ML_OK && make_plan(m, *st, q, n, &plan) == ML_OK)
+        if (device_state(m, &st, &dev) == ML_OK && make_plan(m, *st, q, n, &plan, false) == ML_OK)
           cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, plan.entry.kernel, b,
                                                         plan.smem);
       }

@@ -775,6 +775,7 @@ struct WarpTraj {
       const uint64_t changed = k >= 0 ? md.cmask[k] : ~0ULL;  // unknown: recompute all
 #pragma unroll
       for (int q = 0; q < kRPL; ++q) {
+        if (32 * q >= M) break;
         const int j = lane + 32 * q;
         if (j < M && (md.rmask[j] & changed) != 0ULL) {
           g[q] = g_int(md, j, sl.x);
