@@ -586,8 +586,8 @@ __device__ __forceinline__ bool abs_gt(float a, float b) { return fabsf(a) > fab
 // v t for a net change v: the common changes by one are exact without a product.
 __device__ __noinline__ inline double nu_times_call(int v, double t) { return f64_of_i32(v) * t; }
 __device__ __forceinline__ double nu_times(int v, double t) {
-  return v == 1 ? t : v == -1 ? -t : v == 2 || v == -2 ? (v > 0 ? t + t : -(t + t))
-                                                     : nu_times_call(v, t);
+  return v == 1 ? t : v == -1 ? -t : v == 2 ? 2.0 * t : v == -2 ? -2.0 * t
+                                                                : nu_times_call(v, t);
 }
 __device__ __forceinline__ float nu_times(int v, float t) { return (float)v * t; }
 
@@ -1211,6 +1211,18 @@ struct ImplicitIo {
   float th[MM];
 };
 
+// 1 / b within 2^-44 relative: FP32's reciprocal and one Newton step, two FP64 instructions
+// instead of the division's eight.  For the factors of fast precision's Newton system only:
+// an error of the difference step's or a pivot's reciprocal changes an update by that share
+// of itself, and the iteration ends when the update is below newton_tol of the state, so the
+// solution, fixed by the FP64 residual, does not see it.
+__device__ __forceinline__ double near_recip(double b) {
+  const uint32_t e = ((uint32_t)__double2hiint(b) >> 20) & 0x7ffu;
+  if (e - 923u > 200u) return 1.0 / b;
+  const double y = f64_of_f32(__fdividef(1.f, f32_of_f64(b)));
+  return __fma_rn(y, __fma_rn(-b, y, 1.0), y);
+}
+
 // The implicit leap on tables read at run time: the operations of implicit_solve (kRecip
 // false: the canonical order, a division per Jacobian entry, eliminated row and unknown) or of
 // implicit_leap_wide (true: reciprocals), with loops over the real sizes and arrays in local
@@ -1268,7 +1280,7 @@ __device__ __noinline__ int implicit_leap_rolled(const MDL& md, const long long 
         const double h = fd_h * (f64_abs_gt(y[s], 1.0) ? fabs(y[s]) : 1.0);
         yp[s] = y[s] + h;
         he[s] = yp[s] - y[s];
-        if (kRecip) he[s] = 1.0 / he[s];
+        if (kRecip) he[s] = near_recip(he[s]);
       }
     }
 #pragma unroll 1
@@ -1333,7 +1345,7 @@ __device__ __noinline__ int implicit_leap_rolled(const MDL& md, const long long 
         b[k] = b[piv];
         b[piv] = t;
       }
-      if (kRecip) inv[k] = 1.0 / A[k][k];
+      if (kRecip) inv[k] = near_recip(A[k][k]);
 #pragma unroll 1
       for (int i = k + 1; i < N; ++i) {
         if ((__double_as_longlong(A[i][k]) << 1) == 0) continue;
@@ -1434,12 +1446,11 @@ __device__ __noinline__ int implicit_leap_wide(const MDL& md,
                       ? th[j] * TR::template g_real_deriv<double>(md, j, y, q)
                       : 0.0;
       } else {
-        const double aq = fabs(y[q]);
         double yq[NM];
 #pragma unroll
         for (int s = 0; s < NM; ++s) yq[s] = y[s];
-        yq[q] = y[q] + fd_h * (aq > 1.0 ? aq : 1.0);
-        const double inv_h = 1.0 / (yq[q] - y[q]);
+        yq[q] = y[q] + fd_h * (f64_abs_gt(y[q], 1.0) ? fabs(y[q]) : 1.0);
+        const double inv_h = near_recip(yq[q] - y[q]);
 #pragma unroll
         for (int j = 0; j < MM; ++j)
           Dq[j] = (((nc >> j) & 1u) && md.ord[j][q] != 0)
@@ -1487,7 +1498,7 @@ __device__ __noinline__ int implicit_leap_wide(const MDL& md,
           b[i] = tb;
         }
       }
-      inv_piv[k] = 1.0 / A[k][k];
+      inv_piv[k] = near_recip(A[k][k]);
 #pragma unroll
       for (int i = k + 1; i < NM; ++i) {
         const double l = A[i][k] * inv_piv[k];
@@ -1504,11 +1515,10 @@ __device__ __noinline__ int implicit_leap_wide(const MDL& md,
 #pragma unroll
       for (int rr = 0; rr < i; ++rr) b[rr] -= A[rr][i] * d;
       y[i] += d;
-      dmax = fabs(d) > dmax ? fabs(d) : dmax;
+      dmax = f64_abs_gt(d, dmax) ? fabs(d) : dmax;
     }
 #pragma unroll
-    for (int s = 0; s < NM; ++s) ymax = fabs(y[s]) > ymax ? fabs(y[s]) : ymax;
-    if (!(dmax == dmax)) break;
+    for (int s = 0; s < NM; ++s) ymax = f64_abs_gt(y[s], ymax) ? fabs(y[s]) : ymax;
     if (dmax <= tol * (ymax > 1.0 ? ymax : 1.0)) rc = 0;
   }
   if (rc == 0) {
