@@ -186,16 +186,12 @@ _SRC = ("ncu --metrics gpu__time_duration.sum,smsp__inst_executed.sum,dram__byte
         "--serving-seconds 0 --ncu --shape S --block B "
         "(profiles/k_jit_pool_fast_gene_expression_1M.md)")
 PROFILED = {
-    (2, 6, 128, 1): {"dram_bytes": 262120960 + 209241088, "warp_inst": 123710711486,
-                     "fp64_pipe_pct": 31.60, "source": _SRC},
-    (2, 6, 256, 1): {"dram_bytes": 263632640 + 209561856, "warp_inst": 123667242930,
-                     "fp64_pipe_pct": 31.62, "source": _SRC},
-    (2, 6, 64, 1): {"dram_bytes": 265054208 + 209970688, "warp_inst": 123713090021,
-                    "fp64_pipe_pct": 31.53, "source": _SRC},
-    (2, 1, 256, 1): {"dram_bytes": 271331584 + 210071040, "warp_inst": 188576129640,
-                     "fp64_pipe_pct": 41.24, "source": _SRC},
-    (2, 7, 64, 1): {"dram_bytes": 280494336 + 1490402048, "warp_inst": 135008423302,
-                    "fp64_pipe_pct": 35.65, "source": _SRC},
+    (2, 6, 64, 1): {"dram_bytes": 280674048 + 247611136, "warp_inst": 100004762963,
+                    "fp64_pipe_pct": 12.21, "source": _SRC},
+    (2, 6, 128, 1): {"dram_bytes": 280562432 + 248731648, "warp_inst": 100010507863,
+                     "fp64_pipe_pct": 12.20, "source": _SRC},
+    (2, 7, 64, 1): {"dram_bytes": 300612864 + 2831970048, "warp_inst": 108139420645,
+                    "fp64_pipe_pct": 14.24, "source": _SRC},
 }
 
 

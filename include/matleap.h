@@ -84,7 +84,9 @@ extern "C" {
                                 queue; optionally replayed from a CUDA graph           */
 
 /* ---- kernel shapes ---------------------------------------------------------------- */
-#define ML_SHAPE_AUTO 0   /* thread per trajectory when the model fits, else warp     */
+#define ML_SHAPE_AUTO 0   /* thread per trajectory when the model fits (in reference
+                             precision from some thousand trajectories on: smaller
+                             batches run one per warp, with the same results), else warp */
 #define ML_SHAPE_THREAD 1 /* one trajectory per thread (N <= 8, M <= 16), round-based  */
 #define ML_SHAPE_WARP 2   /* one trajectory per warp (N <= 64, M <= 128)               */
 #define ML_SHAPE_THREAD_OCC 3 /* fast precision only: one trajectory per thread, built
