@@ -125,6 +125,13 @@ __device__ __forceinline__ bool f64_lt_pos(double a, double b) {
   return ((unsigned long long)__double_as_longlong(a) & m) < ub && ub <= inf;
 }
 
+// a <= b for operands that are each in [0, +inf] (not -0) or NaN.
+__device__ __forceinline__ bool f64_le_pos(double a, double b) {
+  const unsigned long long m = 0x7fffffffffffffffULL, inf = 0x7ff0000000000000ULL;
+  const unsigned long long ub = (unsigned long long)__double_as_longlong(b) & m;
+  return ((unsigned long long)__double_as_longlong(a) & m) <= ub && ub <= inf;
+}
+
 // abs(a) > abs(b) (false when a is NaN; b is not NaN).
 __device__ __forceinline__ bool f64_abs_gt(double a, double b) {
   const unsigned long long m = 0x7fffffffffffffffULL, inf = 0x7ff0000000000000ULL;

@@ -210,6 +210,7 @@ struct PrecRef {
   }
   // comparisons of values in [0, +inf] (not -0) or NaN, on the integer pipe
   __device__ static __forceinline__ bool lt(R a, R b) { return f64_lt_pos(a, b); }
+  __device__ static __forceinline__ bool le(R a, R b) { return f64_le_pos(a, b); }
   __device__ static __forceinline__ bool positive(R a) { return f64_lt_pos(0.0, a); }
   __device__ static __forceinline__ bool zero(R a) {
     return (__double_as_longlong(a) << 1) == 0;
@@ -245,6 +246,7 @@ struct PrecFast {
     return k == 0 ? u01_f32(w.w0) : u01_f32(w.w2);
   }
   __device__ static __forceinline__ bool lt(R a, R b) { return a < b; }
+  __device__ static __forceinline__ bool le(R a, R b) { return a <= b; }
   __device__ static __forceinline__ bool positive(R a) { return a > 0.f; }
   __device__ static __forceinline__ bool zero(R a) { return a == 0.f; }
   __device__ static __forceinline__ bool negative(R a) { return a < 0.f; }
@@ -2121,7 +2123,7 @@ struct ThreadLane {
             for (int kk = 0; kk < MM; ++kk)
               if (kk == k) ak = a[kk];
             const R lo = P::lt(a[j], ak) ? a[j] : ak;
-            if (!P::lt(P::pe_delta(A) * lo, fabs(a[j] - ak))) pe |= (1u << j) | (1u << k);
+            if (P::le(fabs(a[j] - ak), P::pe_delta(A) * lo)) pe |= (1u << j) | (1u << k);
           }
         }
         if (pe != 0) {
@@ -2155,11 +2157,11 @@ struct ThreadLane {
         if (P::lt(tau2, tau)) tau = tau2;
         bool at_horizon = false;
         const R rmr = P::of_f64(rm);
-        if (!P::lt(tau, rmr)) {
+        if (P::le(rmr, tau)) {
           tau = rmr;
           at_horizon = true;
         }
-        const bool crit_fire = !P::lt(tau1, tau2) && !P::lt(rmr, tau2);
+        const bool crit_fire = P::le(tau2, tau1) && P::le(tau2, rmr);
         {
           bool over = false;
 #pragma unroll

@@ -1021,7 +1021,7 @@ struct WarpTraj {
               if (k >= 0 && bit(nc, lo_j) && bit(nc, hi_j)) {
                 const R aj = a_s[lo_j], ak = a_s[hi_j];
                 const R lo = P::lt(aj, ak) ? aj : ak;
-                on = !P::lt(P::mul(P::pe_delta(A), lo), fabs(aj - ak));
+                on = P::le(fabs(aj - ak), P::mul(P::pe_delta(A), lo));
               }
             }
             pe[q] = __ballot_sync(0xffffffffu, on);
@@ -1061,11 +1061,11 @@ struct WarpTraj {
           if (P::lt(tau2, tau)) tau = tau2;
           bool at_horizon = false;
           const R rmr = P::of_f64(rem);
-          if (!P::lt(tau, rmr)) {
+          if (P::le(rmr, tau)) {
             tau = rmr;
             at_horizon = true;
           }
-          const bool crit_fire = !P::lt(tau1, tau2) && !P::lt(rmr, tau2);
+          const bool crit_fire = P::le(tau2, tau1) && P::le(tau2, rmr);
           {
             bool over = false;
 #pragma unroll
