@@ -116,12 +116,17 @@ struct WarpTraj {
       const int j = lane + 32 * q;
       if (j < M) s = (q == 0) ? v[q] : s + v[q];
     }
+    if (M > 16) {
+#pragma unroll
+      for (int d = 16; d >= 1; d >>= 1) s = s + __shfl_xor_sync(0xffffffffu, s, d);
+      return s;
+    }
     // a level whose upper lanes are all empty adds zeros: left out (the values are not
     // negative), and the total is then lane 0's
 #pragma unroll
-    for (int d = 16; d >= 1; d >>= 1)
+    for (int d = 8; d >= 1; d >>= 1)
       if (M > d) s = s + __shfl_xor_sync(0xffffffffu, s, d);
-    return M > 16 ? s : __shfl_sync(0xffffffffu, s, 0);
+    return __shfl_sync(0xffffffffu, s, 0);
   }
 
   __device__ static __forceinline__ R g_int(const WarpModel& md, int j, const long long* x) {
