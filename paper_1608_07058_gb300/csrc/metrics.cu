@@ -121,9 +121,12 @@ __global__ void __launch_bounds__(kKlThreads) k_kl(int64_t n_ref, const int64_t*
   const unsigned long long d = (unsigned long long)hi - (unsigned long long)lo;
   const unsigned long long w = d / (unsigned long long)max_bins + 1ull;
   const int nbins = (int)(d / w + 1ull);
+  // the division in 32 bits where range and width both fit (one bin over a range of 2^32 - 1
+  // has a width of 2^32)
+  const bool narrow = ((d | w) >> 32) == 0ull;
   auto bin_of = [&](long long v) {
     const unsigned long long o = (unsigned long long)v - (unsigned long long)lo;
-    return w == 1ull ? (int)o : (d >> 32) == 0ull ? (int)((unsigned)o / (unsigned)w) : (int)(o / w);
+    return w == 1ull ? (int)o : narrow ? (int)((unsigned)o / (unsigned)w) : (int)(o / w);
   };
 
   for_samples(a, n_ref, stride, [&](long long v) { atomicAdd(&bin[bin_of(v)].x, 1u); });

@@ -1,0 +1,30 @@
+"""Accepted inputs at the edges of what the kernels' shortcuts assume, and what shape AUTO's
+choice by the size of the batch may not change: each against the oracle or a direct call."""
+import numpy as np
+import pytest
+
+from paper_1608_07058_gb300 import workloads as W
+from tests.test_gpu_parity import assert_bit_parity, ml, run_gpu, run_oracle  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+
+def torch_of(a):
+    import torch
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+@pytest.mark.parametrize("d", [2**32 - 2, 2**32 - 1, 2**32, 2**33 + 5, 2**62])
+@pytest.mark.parametrize("bins", [1, 2, 3, 4096])
+def test_kl_ranges_around_32_bits(ml, oracle, d, bins):
+    """Pooled ranges around 2^32, where the range fits 32 bits and the width of one bin does
+    not: every value has a bin below max_bins."""
+    rng = np.random.default_rng(3)
+    lo = -(d // 2)
+    a = np.array([lo, lo + d] + [lo + int(u * d) for u in rng.random(398)], np.int64)
+    b = np.array([lo + int(u * u * d) for u in rng.random(300)], np.int64)
+    kl, mean = ml.ml_kl_divergence(torch_of(a.reshape(-1, 1, 1)), torch_of(b.reshape(-1, 1, 1)),
+                                   bins)
+    want, want_mean = oracle.kl_grid(a.reshape(-1, 1, 1), b.reshape(-1, 1, 1), bins)
+    assert np.array_equal(kl.cpu().numpy(), np.asarray(want).reshape(1, 1))
+    assert float(mean) == float(want_mean)
