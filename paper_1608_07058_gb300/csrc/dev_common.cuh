@@ -113,9 +113,13 @@ __device__ __forceinline__ double f64_of_i32(int k) {
   return __hiloint2double((int)(a ? h : 0u), (int)(m << 21));
 }
 
-// a < b for a >= 0 (not -0) and b not NaN: as integers.
-__device__ __forceinline__ bool f64_lt_nn(double a, double b) {
-  return __double_as_longlong(a) < __double_as_longlong(b);
+// t < T for a time t in [0, +inf] or NaN and a horizon T that is not NaN (it may be negative):
+// as unsigned integers with the sign shifted out.  0 inf gives a NaN whose sign is set, which
+// as a signed integer lies below every T; the absolute value may be an FP64 instruction and
+// leave that sign.
+__device__ __forceinline__ bool before_horizon(double t, double T) {
+  const long long bT = __double_as_longlong(T);
+  return bT > 0 && ((unsigned long long)__double_as_longlong(t) << 1) < ((unsigned long long)bT << 1);
 }
 
 // a < b for operands that are each in [0, +inf] (not -0) or NaN.

@@ -1878,7 +1878,7 @@ struct ThreadLane {
         a0 = reaction_sum<MM, R, P::kRef>(a);
         const double dt = wait[i] / a0;
         tn = tn + dt;
-        ok = ok && P::positive(a0) && !f64_lt_nn(T, tn);
+        ok = ok && P::positive(a0) && !f64_lt_pos(T, tn);
 #pragma unroll
         for (int j = 0; j < MM; ++j)
           if (TT::g_owner(j) == j) Gn[j] = Gn[j] + (double)g[j] * dt;
@@ -1994,7 +1994,7 @@ struct ThreadLane {
           if constexpr (P::kRef) {
             const R dt = -P::log(P::u(w, 0)) / a0;
             const double tn = t + (double)dt;
-            if (f64_lt_nn(T, tn)) {
+            if (f64_lt_pos(T, tn)) {
               to_horizon = burst_over = true;
               break;
             }
@@ -2055,7 +2055,7 @@ struct ThreadLane {
   __device__ __forceinline__ void eval_phase(const Model& md, const SimArgs& A) {
     const uint32_t k0 = (uint32_t)A.seed, k1 = (uint32_t)(A.seed >> 32);
     const uint32_t Mr = (uint32_t)A.M;  // stream numbering uses the real M
-    if (!f64_lt_nn(t, T)) {
+    if (!before_horizon(t, T)) {
       mode = kDone;
       return;
     }

@@ -74,11 +74,12 @@ __device__ inline WarpSlab carve_slab(char* p, int N, int M, int rbytes, int lby
   return s;
 }
 
-// Comparisons of the Newton system on the integer pipe: a > b for b >= -1 (a not negative;
-// false when a is NaN), equality of values that are not NaN, zero.
+// Comparisons of the Newton system on the integer pipe: a > b where each is not negative or
+// -1 (no row) and b is not NaN, false when a is NaN of either sign; equality of values that
+// are not NaN; zero.
 __device__ __forceinline__ bool pivot_gt(double a, double b) {
   const long long ua = __double_as_longlong(a);
-  return ua > __double_as_longlong(b) && ua <= 0x7ff0000000000000LL;
+  return ua > __double_as_longlong(b) && ((unsigned long long)ua << 1) <= 0xffe0000000000000ULL;
 }
 __device__ __forceinline__ bool pivot_gt(float a, float b) { return a > b; }
 __device__ __forceinline__ bool same_bits(double a, double b) {
@@ -917,7 +918,7 @@ struct WarpTraj {
                        __shfl_sync(0xffffffffu, wl.w3, b & 31)};
         const R dt = __shfl_sync(0xffffffffu, wait_l, b & 31) / a0;
         const double tn = t + (double)dt;
-        if (f64_lt_nn(T, tn)) {
+        if (f64_lt_pos(T, tn)) {
           const double rem = T - t;
 #pragma unroll
           for (int q = 0; q < kRPL; ++q) G[q] = G[q] + (double)g[q] * rem;
@@ -950,7 +951,7 @@ struct WarpTraj {
 
     const R eps = P::eps(A);
     for (;;) {
-      if (!f64_lt_nn(t, T)) break;
+      if (!before_horizon(t, T)) break;
       if ((long long)step >= A.max_steps) {
         status |= ML_ST_STEP_LIMIT;
         break;

@@ -28,3 +28,29 @@ def test_kl_ranges_around_32_bits(ml, oracle, d, bins):
     want, want_mean = oracle.kl_grid(a.reshape(-1, 1, 1), b.reshape(-1, 1, 1), bins)
     assert np.array_equal(kl.cpu().numpy(), np.asarray(want).reshape(1, 1))
     assert float(mean) == float(want_mean)
+
+
+@pytest.mark.parametrize("mode", [0, 2])
+@pytest.mark.parametrize("kw", [dict(shape=1), dict(shape=2), dict(shape=4), dict(shape=6, form=1),
+                                dict(shape=1, specialize=1), dict(shape=6, form=1, specialize=1)])
+def test_infinite_rate_of_an_absent_reactant(ml, oracle, mode, kw):
+    """theta = +inf is accepted (not negative, not NaN); with g = 0 the propensity and a0 are
+    NaN.  An SSA firing's time is then NaN: it is not past T, fires, and ends the trajectory
+    after its burst, in every driver as in the oracle."""
+    crn = W._crn("absent", 2, [({0: 1}, {}, 1.0), ({}, {1: 1}, 5.0), ({1: 1}, {}, 1.0)])
+    n = 70
+    theta = np.tile([np.inf, 5.0, 1.0], (n, 1))
+    T = np.linspace(0.1, 2.0, n)
+    args = dict(theta=theta, seed=21, mode=mode, max_steps=50)
+    o = run_oracle(oracle, crn, n, [0, 10], T, **args)
+    if mode == 2:
+        assert np.isnan(o["G"]).all() and (o["counters"][:, 2] == 100).all()
+    g = run_gpu(ml, crn, n, [0, 10], T, **args, **kw)
+    for key in ("X", "r", "status", "counters"):
+        assert np.array_equal(g[key], o[key]), key
+    assert np.array_equal(g["G"], o["G"], equal_nan=True)
+    if mode == 2:  # fast precision: the same firings
+        f = run_gpu(ml, crn, n, [0, 10], T, precision=ml.ML_PREC_FAST_FP32, **args, **kw)
+        for key in ("X", "r", "status", "counters"):
+            assert np.array_equal(f[key], o[key]), key
+        assert np.isnan(f["G"]).all()
