@@ -381,36 +381,40 @@ int device_state(ml_model* m, DeviceState** out, int* device) {
   return ML_OK;
 }
 
-int ensure_tables(ml_model* m, DeviceState& st, int shape, int variant) {
-  if (shape == ML_SHAPE_THREAD) {
-    if (!st.thread_tables[variant]) {
-      std::vector<uint8_t> b = thread_tables(variant, *m);
-      void* d = nullptr;
-      ML_CUDA_TRY(cudaMalloc(&d, b.size()));
-      cudaError_t e = cudaMemcpy(d, b.data(), b.size(), cudaMemcpyHostToDevice);
-      if (e != cudaSuccess) {
-        cudaFree(d);
-        return cuda_fail(e, "upload thread tables");
-      }
-      st.thread_tables[variant] = d;
-    }
+int upload(const std::vector<uint8_t>& b, void** out, const char* what) {
+  void* d = nullptr;
+  ML_CUDA_TRY(cudaMalloc(&d, b.size()));
+  cudaError_t e = cudaMemcpy(d, b.data(), b.size(), cudaMemcpyHostToDevice);
+  if (e != cudaSuccess) {
+    cudaFree(d);
+    return cuda_fail(e, what);
   }
-  // The warp kernel's tables too where the model fits both, and its reference builds loaded:
-  // shape AUTO takes one or the other by the size of the batch, and a call that a program
-  // captures after warming up with another size must not be the one that allocates.
-  if (!st.warp_tables && (shape == ML_SHAPE_WARP || warp_fits(*m))) {
+  *out = d;
+  return ML_OK;
+}
+
+// The tables of both kernel kinds where the model fits both, and the reference builds of both
+// that shape AUTO may take loaded: AUTO chooses by the size of the batch, and a call that a
+// program captures after warming up with another size must not be the one that allocates or
+// loads.  Two small uploads at the first call.
+int ensure_tables(ml_model* m, DeviceState& st, int variant) {
+  const bool thread = variant >= 0, warp = warp_fits(*m);
+  const bool first = (thread && !st.thread_tables[variant]) || (warp && !st.warp_tables);
+  if (thread && !st.thread_tables[variant]) {
+    int rc = upload(thread_tables(variant, *m), &st.thread_tables[variant], "upload thread tables");
+    if (rc != ML_OK) return rc;
+  }
+  if (warp && !st.warp_tables) {
+    int rc = upload(warp_tables(*m), &st.warp_tables, "upload warp tables");
+    if (rc != ML_OK) return rc;
+  }
+  if (first && thread && warp) {
+    const mlk::KernelEntry entries[] = {
+        thread_entry(ML_PREC_REF_FP64, variant), thread_seq_grid_entry(ML_PREC_REF_FP64, variant),
+        warp_entry(ML_PREC_REF_FP64), warp_grid_entry(ML_PREC_REF_FP64)};
     cudaFuncAttributes fa;
-    ML_CUDA_TRY(cudaFuncGetAttributes(&fa, warp_entry(ML_PREC_REF_FP64).kernel));
-    ML_CUDA_TRY(cudaFuncGetAttributes(&fa, warp_grid_entry(ML_PREC_REF_FP64).kernel));
-    std::vector<uint8_t> b = warp_tables(*m);
-    void* d = nullptr;
-    ML_CUDA_TRY(cudaMalloc(&d, b.size()));
-    cudaError_t e = cudaMemcpy(d, b.data(), b.size(), cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) {
-      cudaFree(d);
-      return cuda_fail(e, "upload warp tables");
-    }
-    st.warp_tables = d;
+    for (const auto& e : entries)
+      if (e.kernel) ML_CUDA_TRY(cudaFuncGetAttributes(&fa, e.kernel));
   }
   if (!st.queues) {
     void* q = nullptr;
@@ -452,6 +456,9 @@ int jit_entry(ml_model* m, int variant, int precision, int driver, bool occ,
     ML_CUDA_TRY(cudaLibraryLoadData(&jk.lib, cubin.data(), nullptr, nullptr, 0, nullptr,
                                     nullptr, 0));
     cudaError_t e = cudaLibraryGetKernel(&jk.kernel, jk.lib, "ml_jit_kernel");
+    cudaFuncAttributes fa;  // loads it on this device
+    if (e == cudaSuccess)
+      e = cudaFuncGetAttributes(&fa, reinterpret_cast<const void*>(jk.kernel));
     if (e != cudaSuccess) {
       cudaLibraryUnload(jk.lib);
       return cuda_fail(e, "specialized kernel lookup");
@@ -507,11 +514,12 @@ int make_plan(ml_model* m, DeviceState& st, const ml_sim_params& p, int64_t n_tr
   const int variant = thread_variant_for(*m);
   auto tk = st.tuned.find({p.precision, p.form});
   const Tuned* tuned = tk == st.tuned.end() ? nullptr : &tk->second;
+  bool by_size = false;  // the warp kernel for this size of batch, the thread kernel for larger
   if (shape == ML_SHAPE_AUTO) {
-    const bool small = p.precision == ML_PREC_REF_FP64 && warp_fits(*m) &&
-                       n_traj <= ref_warp_limit(*m, st, p, ragged);
+    by_size = !(tuned && tuned->shape) && variant >= 0 && p.precision == ML_PREC_REF_FP64 &&
+              warp_fits(*m) && n_traj <= ref_warp_limit(*m, st, p, ragged);
     shape = tuned && tuned->shape ? tuned->shape
-                                  : (variant >= 0 && !small ? ML_SHAPE_THREAD : ML_SHAPE_WARP);
+                                  : (variant >= 0 && !by_size ? ML_SHAPE_THREAD : ML_SHAPE_WARP);
   }
   const int req_shape = shape;
   // a call with time-grid output runs the grid build of the sequential driver (the
@@ -546,8 +554,15 @@ int make_plan(ml_model* m, DeviceState& st, const ml_sim_params& p, int64_t n_tr
   } else if (!entry.kernel || !entry.launch) {
     return fail(ML_ERR_UNSUPPORTED, "no kernel built for this shape and precision");
   }
-  int rc = ensure_tables(m, st, shape, variant);
+  int rc = ensure_tables(m, st, variant);
   if (rc != ML_OK) return rc;
+  if (by_size && p.specialize && !grid_out) {
+    // a larger call of the same kind runs the kernel compiled for the model: compiled and
+    // loaded here too, so that a warm-up of any size covers it
+    mlk::KernelEntry larger{};
+    rc = jit_entry(m, variant, p.precision, mlk::kJitRounds, false, &larger);
+    if (rc != ML_OK) return rc;
+  }
   plan->shape = shape;
   plan->jit = jit;
   plan->occ = occ;

@@ -54,3 +54,35 @@ def test_infinite_rate_of_an_absent_reactant(ml, oracle, mode, kw):
         for key in ("X", "r", "status", "counters"):
             assert np.array_equal(f[key], o[key]), key
         assert np.isnan(f["G"]).all()
+
+
+@pytest.mark.parametrize("first,then", [(100, 6000), (6000, 100)])
+@pytest.mark.parametrize("specialize", [0, 1])
+@pytest.mark.parametrize("grid", [False, True])
+def test_warm_up_of_any_size_covers_a_captured_call(ml, first, then, specialize, grid):
+    """Shape AUTO takes another kernel for another size of the batch: a call captured after
+    one warm-up of a size on the other side of the line allocates and loads nothing."""
+    import torch
+    crn = W.dimerisation()
+    x0 = torch.tensor([400, 798, 0], device="cuda")
+    T = torch.full((1,), 0.02, dtype=torch.float64, device="cuda")
+    t_obs = torch.tensor([0.01, 0.02], dtype=torch.float64, device="cuda")
+    params = ml.ml_default_params(form=ml.ML_FORM_PERSISTENT, specialize=specialize)
+
+    def call(model, n):
+        if grid:
+            return ml.ml_simulate_grid(model, n, x0, T, t_obs, params=params, seed=5)
+        return ml.ml_simulate(model, n, x0, T, params=params, seed=5)
+
+    model = ml.model_from_crn(crn)
+    call(model, first)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        out = call(model, then)
+    graph.replay()
+    torch.cuda.synchronize()
+    want = call(ml.model_from_crn(crn), then)
+    torch.cuda.synchronize()
+    for key in want:
+        assert torch.equal(out[key], want[key]), key
