@@ -52,11 +52,13 @@ __device__ __forceinline__ Signed52 signed52(uint32_t hi, uint32_t lo) {
 // 3 d (-y^4/4 + y^5/5 - ...): the large terms cancel before they are formed.  For |y| < 1/4
 // the series to y^11 (relative error below 1e-5); else the logarithm, where d <= 16 z^2 / 9 <
 // 140 (|z| < 8.7 from 52-bit uniforms) keeps its FP32 error 3 d 4e-7 below 2e-4; next to
-// y = -1, where the rounding of y counts for more, it does not tell.
+// y = -1, where the rounding of y counts for more, it does not tell.  The FP64 test adds terms
+// of size d, so it is itself off by up to about 4 d 2^-53: below the margin by a factor of 30
+// up to d = 2^36; from there on (and for NaN) it does not tell either.
 __device__ __forceinline__ int gamma_estimate(float u, float y, float d) {
   const float y2 = y * y;
   float t;
-  if (y < -0.999f) return 0;
+  if (y < -0.999f || !(d < 0x1p36f)) return 0;
   if (fabsf(y) < 0.25f) {
     float q = 1.f / 11.f;
     q = q * y - 0.1f;

@@ -86,3 +86,16 @@ def test_warm_up_of_any_size_covers_a_captured_call(ml, first, then, specialize,
     torch.cuda.synchronize()
     for key in want:
         assert torch.equal(out[key], want[key]), key
+
+
+def test_posterior_huge_shapes(ml, oracle):
+    """Shapes on both sides of the FP32 estimate's range and far beyond it, where the FP64
+    acceptance test is its own rounding noise: every draw is the oracle's."""
+    alpha = np.array([6.8e10, 6.9e10, 1e12, 1e13, 1e14, 1e15, 1e17, 1e300])
+    n, M = 4000, alpha.size
+    beta, r, G = np.ones(M), np.zeros((n, M), np.int64), np.zeros((n, M))
+    th, st = ml.ml_posterior_sample(*(torch_of(a) for a in (alpha, beta, r, G)), seed=17)
+    want, want_st = oracle.posterior_sample(alpha, beta, r, G, seed=17, traj_id_base=0)
+    differ = (th.cpu().numpy() != want).sum(0)
+    assert not differ.any(), dict(zip(alpha, differ))
+    assert np.array_equal(st.cpu().numpy().astype(np.uint32), want_st)
