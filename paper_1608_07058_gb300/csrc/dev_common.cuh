@@ -122,6 +122,13 @@ __device__ __forceinline__ bool before_horizon(double t, double T) {
   return bT > 0 && ((unsigned long long)__double_as_longlong(t) << 1) < ((unsigned long long)bT << 1);
 }
 
+// tn > T for a time tn in [0, +inf] (not -0) or NaN of either sign and a horizon T > 0: false
+// for a NaN (a set sign makes it negative).
+__device__ __forceinline__ bool past_horizon(double tn, double T) {
+  const long long bt = __double_as_longlong(tn);
+  return bt > __double_as_longlong(T) && bt <= 0x7ff0000000000000LL;
+}
+
 // a < b for operands that are each in [0, +inf] (not -0) or NaN.
 __device__ __forceinline__ bool f64_lt_pos(double a, double b) {
   const unsigned long long m = 0x7fffffffffffffffULL, inf = 0x7ff0000000000000ULL;

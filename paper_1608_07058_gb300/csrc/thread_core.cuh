@@ -1878,7 +1878,7 @@ struct ThreadLane {
         a0 = reaction_sum<MM, R, P::kRef>(a);
         const double dt = wait[i] / a0;
         tn = tn + dt;
-        ok = ok && P::positive(a0) && !f64_lt_pos(T, tn);
+        ok = ok && P::positive(a0) && !past_horizon(tn, T);
 #pragma unroll
         for (int j = 0; j < MM; ++j)
           if (TT::g_owner(j) == j) Gn[j] = Gn[j] + (double)g[j] * dt;
@@ -1994,7 +1994,7 @@ struct ThreadLane {
           if constexpr (P::kRef) {
             const R dt = -P::log(P::u(w, 0)) / a0;
             const double tn = t + (double)dt;
-            if (f64_lt_pos(T, tn)) {
+            if (past_horizon(tn, T)) {
               to_horizon = burst_over = true;
               break;
             }

@@ -918,7 +918,7 @@ struct WarpTraj {
                        __shfl_sync(0xffffffffu, wl.w3, b & 31)};
         const R dt = __shfl_sync(0xffffffffu, wait_l, b & 31) / a0;
         const double tn = t + (double)dt;
-        if (f64_lt_pos(T, tn)) {
+        if (past_horizon(tn, T)) {
           const double rem = T - t;
 #pragma unroll
           for (int q = 0; q < kRPL; ++q) G[q] = G[q] + (double)g[q] * rem;
