@@ -1213,16 +1213,16 @@ struct ImplicitIo {
   float th[MM];
 };
 
-// 1 / b within 2^-44 relative: FP32's reciprocal and one Newton step, two FP64 instructions
-// instead of the division's eight.  For the factors of fast precision's Newton system only:
-// an error of the difference step's or a pivot's reciprocal changes an update by that share
-// of itself, and the iteration ends when the update is below newton_tol of the state, so the
-// solution, fixed by the FP64 residual, does not see it.
+// 1 / b within 0.501 ulp: with FP32's reciprocal y (within 2^-21) and e = 1 - b y, the sum
+// y + y (e + e^2) misses 1 / b by e^3 before its rounding, so it is the rounded quotient but
+// for at most one b in a thousand (then its neighbour).  Three FP64 instructions; used where
+// fast precision's Newton system divides by a difference step or a pivot.
 __device__ __forceinline__ double near_recip(double b) {
-  const uint32_t e = ((uint32_t)__double2hiint(b) >> 20) & 0x7ffu;
-  if (e - 923u > 200u) return 1.0 / b;
+  const uint32_t ex = ((uint32_t)__double2hiint(b) >> 20) & 0x7ffu;
+  if (ex - 923u > 200u) return 1.0 / b;
   const double y = f64_of_f32(__fdividef(1.f, f32_of_f64(b)));
-  return __fma_rn(y, __fma_rn(-b, y, 1.0), y);
+  const double e = __fma_rn(-b, y, 1.0);
+  return __fma_rn(y, __fma_rn(e, e, e), y);
 }
 
 // The implicit leap on tables read at run time: the operations of implicit_solve (kRecip

@@ -1,5 +1,7 @@
 """Accepted inputs at the edges of what the kernels' shortcuts assume, and what shape AUTO's
 choice by the size of the batch may not change: each against the oracle or a direct call."""
+import os
+
 import numpy as np
 import pytest
 
@@ -99,3 +101,19 @@ def test_posterior_huge_shapes(ml, oracle):
     differ = (th.cpu().numpy() != want).sum(0)
     assert not differ.any(), dict(zip(alpha, differ))
     assert np.array_equal(st.cpu().numpy().astype(np.uint32), want_st)
+
+
+def test_reciprocals_of_the_fast_newton_system(tmp_path):
+    """Before its last rounding the reciprocal is within 2^-63 (the third power of FP32's
+    2^-21), so it may differ from the division's only where 1/b lies within 2^-10 ulp of a
+    midpoint: at most 2^-9 of the values, by one unit in the last place."""
+    import subprocess
+    from paper_1608_07058_gb300 import build as B
+    exe = str(tmp_path / "recip_check")
+    src = os.path.join(os.path.dirname(os.path.abspath(__file__)), "recip_check.cu")
+    cmd = [B._nvcc(), *B.ARCH, "-O2", "-std=c++17", "-I", B.CSRC, "-I", B.INCLUDE, src, "-o", exe]
+    assert subprocess.run(cmd, capture_output=True, text=True).returncode == 0
+    res = subprocess.run([exe], capture_output=True, text=True, timeout=120)
+    assert res.returncode == 0
+    n, differ, ulps = map(int, res.stdout.split())
+    assert n == 2**24 and differ <= n * 2**-9 and ulps <= 1
