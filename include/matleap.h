@@ -85,8 +85,9 @@ extern "C" {
 
 /* ---- kernel shapes ---------------------------------------------------------------- */
 #define ML_SHAPE_AUTO 0   /* thread per trajectory when the model fits (in reference
-                             precision from some thousand trajectories on: smaller
-                             batches run one per warp, with the same results), else warp */
+                             precision, without a tuned shape, batches up to 1 to 9
+                             times the resident warps run one per warp, with the same
+                             results: 8 warps per SM, fewer by ctas_per_sm), else warp */
 #define ML_SHAPE_THREAD 1 /* one trajectory per thread (N <= 8, M <= 16), round-based  */
 #define ML_SHAPE_WARP 2   /* one trajectory per warp (N <= 64, M <= 128)               */
 #define ML_SHAPE_THREAD_OCC 3 /* fast precision only: one trajectory per thread, built
@@ -174,8 +175,11 @@ typedef struct {
                                a second, and loads it on the device), 0 = the
                                precompiled kernels that read the tables at run time.
                                Results are identical (reference precision: bitwise).
-                               Ignored by the warp shape, time-grid calls and
-                               ml_simulate_noalloc; the server passes it on.          */
+                               Ignored by the warp shape (which shape AUTO takes for
+                               small reference-precision batches; they still compile
+                               the kernel, so that any first call is a warm-up for
+                               larger ones), time-grid calls and ml_simulate_noalloc;
+                               the server passes it on.                               */
 } ml_sim_params;
 
 /* Fills *p with the defaults above.  Returns ML_ERR_ARG if p is NULL. */

@@ -74,6 +74,7 @@ struct DeviceState {
   unsigned long long* queues = nullptr;  // kQueueSlots counters
   unsigned next_slot = 0;
   int sm_count = 0;
+  int warps_per_sm = 0;  // resident at once, of the reference warp kernel on this model
   std::map<std::pair<int, int>, GraphCache> graphs;  // (precision, shape/variant)
   std::map<std::pair<int, int>, Tuned> tuned;        // (precision, form)
   // host-path workspace
@@ -490,20 +491,50 @@ struct Plan {
 
 // Reference precision: the largest batch that shape AUTO runs one trajectory per warp, where
 // a trajectory's FP64 operations are spread over the lanes, although the model fits one
-// thread (both kernels give the same bits).  Measured on 152 SMs, thread / warp kernel in ms:
-// equal horizons and rate constants, immigration-death 1,216: 5.8 / 4.3, 2,000: 6.3 / 8.0,
-// dimerisation 1,216: 1.9 / 1.2, 4,000: 3.6 / 4.4 -- up to the warps resident at once (8 per
-// SM); their own horizons and rate constants per trajectory, where the longest ones decide:
-// immigration-death 4,000: 16.9 / 15.5, 8,000: 15.2 / 17.2, dimerisation 4,000: 13.5 / 9.5,
-// 8,000: 15.9 / 16.9, gene expression (6 reactions) 4,000: 386 / 194, 10,007: 527 / 357,
-// 16,000: 580 / 437 -- up to 4 of them per warp, 12 with more than 4 reactions.  Kernels
-// compiled for the model are about 1.5 times as fast: 1 and 4 (gene expression 3,000: 275 / 197).
-int64_t ref_warp_limit(const ml_model& m, const DeviceState& st, const ml_sim_params& p,
-                       bool ragged) {
-  const int64_t resident = (int64_t)st.sm_count * 8;
-  if (!ragged) return resident;
-  const bool large = m.M > 4;
-  return resident * (p.specialize ? (large ? 4 : 1) : (large ? 12 : 4));
+// thread (both kernels give the same bits).  A warp takes one trajectory at a time, so the
+// limit is in units of the warps resident at once (8 per SM unless the caller asks for fewer
+// CTAs).  Whether a network gains follows from its paths (a lane of the thread kernel waits
+// for lanes in another phase: most where leaps and bursts alternate, least where all are in
+// bursts), which a call does not know; so a line lies near where the geometric mean of warp
+// time over thread time reaches 1.  Measured on 152 SMs (a unit is 1,216 trajectories), 19
+// workloads on 13 networks, geometric mean (range):
+//   equal trajectories      1 unit 0.52 (0.20-0.97), 2 units 0.81 (0.36-1.38), 4 units up to
+//                           3.1: past one wave of trajectories the loss is steep, so 1;
+//   own rate constants and horizons, where the longest trajectories decide:
+//     persistent  <= 4 reactions  4 units 0.92 (0.75-1.11), 6.6 1.10 (0.91-1.42)
+//                 5, 6 reactions  4 units 0.76 (0.50-1.19), 9 1.00 (0.57-1.85), 12 1.24
+//                 8 x 16 kernel   4 units 0.69 (0.52-1.03), 6.6 1.04 (0.81-1.55)
+//     plain (no refill of a warp)
+//                 <= 4 reactions  3 units 0.92 (0.74-1.32), 4 1.07
+//                 more            4 units 0.84 (0.50-1.36), 6.6 1.11 (0.57-2.02)
+//     thread kernel compiled for the model
+//                                 2 units 0.81 (0.57-1.14), 3 0.99 (0.79-1.22);
+//   own rate constants and one horizon, or the reverse
+//                           1 unit 0.51 (0.18-0.81), 2 units 0.69 (0.29-1.25): 1 too.
+// Gene expression, 10,007 own rate constants and horizons: 530 ms on threads, 352 on warps;
+// Lotka-Volterra with births, the furthest the other way: 35 and 62.
+int64_t ref_warp_limit(const ml_model& m, DeviceState& st, const ml_sim_params& p, bool ragged,
+                       bool grid_out) {
+  const bool persistent = p.form == ML_FORM_PERSISTENT;
+  if (st.warps_per_sm == 0) {
+    int ctas = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+            &ctas, warp_entry(ML_PREC_REF_FP64).kernel, 128,
+            mlk::warp_smem_bytes(4, m.N, m.M, ML_PREC_REF_FP64, false)) != cudaSuccess) {
+      cudaGetLastError();
+      ctas = 0;
+    }
+    st.warps_per_sm = std::max(1, 4 * ctas);
+  }
+  int per_sm = st.warps_per_sm;
+  if (persistent && p.ctas_per_sm)
+    per_sm = std::min(per_sm, p.ctas_per_sm * (p.block_size ? p.block_size : 128) / 32);
+  if (!ragged) return (int64_t)st.sm_count * per_sm;
+  // rows: kernels for up to 4 reactions, for 5 and 6 (3 species), 8 x 16
+  static constexpr int kUnits[3][2] = {{3, 4}, {5, 9}, {5, 6}};  // plain, persistent
+  const int row = mlk::kThreadM[m.thread_variant] <= 4 ? 0 : mlk::kThreadM[m.thread_variant] <= 6 ? 1 : 2;
+  const int units = p.specialize && !grid_out ? 2 : kUnits[row][persistent ? 1 : 0];
+  return (int64_t)st.sm_count * per_sm * units;
 }
 
 // Chooses the kernel and launch shape for one call (model lock held).  ragged: the call gives
@@ -517,7 +548,7 @@ int make_plan(ml_model* m, DeviceState& st, const ml_sim_params& p, int64_t n_tr
   bool by_size = false;  // the warp kernel for this size of batch, the thread kernel for larger
   if (shape == ML_SHAPE_AUTO) {
     by_size = !(tuned && tuned->shape) && variant >= 0 && p.precision == ML_PREC_REF_FP64 &&
-              warp_fits(*m) && n_traj <= ref_warp_limit(*m, st, p, ragged);
+              warp_fits(*m) && n_traj <= ref_warp_limit(*m, st, p, ragged, grid_out);
     shape = tuned && tuned->shape ? tuned->shape
                                   : (variant >= 0 && !by_size ? ML_SHAPE_THREAD : ML_SHAPE_WARP);
   }
