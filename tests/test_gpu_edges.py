@@ -6,6 +6,7 @@ import numpy as np
 import pytest
 
 from paper_1608_07058_gb300 import workloads as W
+from tests.test_gpu_grid import assert_grid_parity, run_gpu_grid, run_oracle_grid
 from tests.test_gpu_parity import assert_bit_parity, ml, run_gpu, run_oracle  # noqa: F401
 
 pytestmark = pytest.mark.gpu
@@ -117,3 +118,75 @@ def test_reciprocals_of_the_fast_newton_system(tmp_path):
     assert res.returncode == 0
     n, differ, ulps = map(int, res.stdout.split())
     assert n == 2**24 and differ <= n * 2**-9 and ulps <= 1
+
+
+# Reference precision with the shape named, so that both kernels run whatever shape AUTO would
+# choose for these sizes: (shape, compiled for the model).
+KERNELS = [(1, 0), (1, 1), (2, 0)]
+
+
+@pytest.mark.parametrize("shape,specialize", KERNELS)
+@pytest.mark.parametrize("form", [0, 1])
+@pytest.mark.parametrize("n", [1, 31, 33, 257, 607, 609])
+def test_reference_tiny_batches_per_shape(ml, oracle, shape, specialize, form, n):
+    """Around a warp and around the batch that is spread one trajectory to a warp (608 on 152
+    SMs), per-trajectory rate constants and horizons (some zero)."""
+    crn = W.gene_expression()
+    rng = np.random.default_rng(n)
+    theta = rng.gamma(2.0, crn.rates / 2.0, size=(n, 6))
+    T = rng.uniform(0.0, 6.0, n)
+    T[::7] = 0.0
+    g = run_gpu(ml, crn, n, [1, 2, 20], T, theta, seed=8, shape=shape, specialize=specialize,
+                form=form)
+    o = run_oracle(oracle, crn, n, [1, 2, 20], T, theta, seed=8)
+    assert_bit_parity(g, o, f"n={n}")
+
+
+@pytest.mark.parametrize("shape,specialize", KERNELS)
+def test_reference_inputs_per_trajectory_per_shape(ml, oracle, shape, specialize):
+    """Per-trajectory x0, T and theta with an id offset, and the gene-expression batch."""
+    kw = dict(shape=shape, specialize=specialize)
+    w = W.config(1, n_traj=700)
+    rng = np.random.default_rng(2)
+    x0 = rng.integers(0, 500, size=(700, 3))
+    T = rng.uniform(0.0, 0.3, size=700)
+    T[:5] = 0.0
+    theta = np.abs(w.crn.rates * rng.gamma(2.0, 0.5, size=(700, 4)))
+    args = dict(seed=2**40 + 9, base=123456)
+    assert_bit_parity(run_gpu(ml, w.crn, 700, x0, T, theta, **args, **kw),
+                      run_oracle(oracle, w.crn, 700, x0, T, theta, **args), "per-trajectory")
+    w = W.config(2, n_traj=400)
+    assert_bit_parity(run_gpu(ml, w.crn, 400, w.x0, w.T, w.theta, seed=3, **kw),
+                      run_oracle(oracle, w.crn, 400, w.x0, w.T, w.theta, seed=3), "gene")
+
+
+@pytest.mark.parametrize("shape", [1, 2])
+def test_reference_forms_per_shape(ml, shape):
+    """Plain, persistent, graph and host calls of one shape give the same results."""
+    w = W.config(2, n_traj=1500)
+    T = w.T * 0.2
+    model = ml.model_from_crn(w.crn)
+    calls = [dict(), dict(form=1, block_size=64, ctas_per_sm=2), dict(form=1, use_graph=1)]
+    if shape == 1:
+        calls += [dict(specialize=1), dict(form=1, use_graph=1, specialize=1)]
+    runs = [run_gpu(ml, w.crn, w.n_traj, w.x0, T, w.theta, seed=4, model=model, shape=shape, **kw)
+            for kw in calls]
+    host = ml.ml_simulate_host(model, w.n_traj, w.x0, T, w.theta,
+                               params=ml.ml_default_params(shape=shape, max_steps=200_000), seed=4)
+    host["status"] = host["status"].astype(np.uint32)
+    for other in runs[1:] + [host]:
+        for key in runs[0]:
+            assert np.array_equal(runs[0][key], other[key]), key
+
+
+@pytest.mark.parametrize("shape", [1, 2])
+def test_reference_time_grid_per_shape(ml, oracle, shape):
+    """Per-trajectory horizons below, at and above grid points, and gene expression."""
+    rng = np.random.default_rng(4)
+    for crn, x0, T, grid in ((W.dimerisation(), [400, 798, 0], rng.uniform(0.01, 0.3, 1000),
+                              [0.0, 0.05, 0.1, 0.2, 0.25]),
+                             (W.gene_expression(), [1, 2, 20], rng.uniform(1.0, 20.0, 300),
+                              [0.5, 5.0, 5.0, 12.0])):
+        g = run_gpu_grid(ml, crn, T.size, x0, T, grid, seed=2, shape=shape)
+        o = run_oracle_grid(oracle, crn, T.size, x0, T, grid, seed=2)
+        assert_grid_parity(g, o, crn.name)
