@@ -230,7 +230,6 @@ struct PrecRef {
     return refmath::log_factorial_ref(k);
   }
   __device__ static __forceinline__ R sqrt(R x) { return ::sqrt(x); }
-  __device__ static __forceinline__ R log1p(R x) { return ::log1p(x); }  // unused
   __device__ static __forceinline__ R inf() {
     return __longlong_as_double(0x7ff0000000000000LL);
   }
@@ -325,20 +324,21 @@ __device__ __noinline__ bool ptrs_accept(typename P::R mu, typename P::R a, type
   using R = typename P::R;
   const R inv_alpha = R(1.1239) + R(1.1328) / (b - R(3.4));
   const R lhs = (P::log(V) + P::log(inv_alpha)) - P::log(a / (us * us) + b);
-  R rhs;
-  if (P::kRef || lt_pos(kd, R(10))) {
-    const R loglam = P::log(mu);
-    rhs = (-mu + kd * loglam) - P::lfact(count_of(kd));
-  } else {
-    // log of the Poisson pmf without cancellation: with z = k + 1 and Stirling's series
-    // for log Gamma(z), -mu + k log mu - log k! =
-    //   (z - mu) + (z - 1) log1p((mu - z)/z) - log(z)/2 - log(2 pi)/2 - 1/(12 z) + 1/(360 z^3)
-    const R z = kd + R(1);
-    const R iz = R(1) / z;
-    rhs = ((z - mu) + (z - R(1)) * P::log1p((mu - z) * iz)) - R(0.5) * P::log(z) -
-          R(0.91893853320467274178) - iz * (R(1) / R(12) - (iz * iz) * (R(1) / R(360)));
+  if constexpr (!P::kRef) {
+    if (!lt_pos(kd, R(10))) {
+      // log of the Poisson pmf without cancellation: with z = k + 1 and Stirling's series
+      // for log Gamma(z), -mu + k log mu - log k! =
+      //   (z - mu) + (z - 1) log1p((mu - z)/z) - log(z)/2 - log(2 pi)/2 - 1/(12 z) + 1/(360 z^3)
+      const R z = kd + R(1);
+      const R iz = R(1) / z;
+      const R rhs = ((z - mu) + (z - R(1)) * P::log1p((mu - z) * iz)) - R(0.5) * P::log(z) -
+                    R(0.91893853320467274178) -
+                    iz * (R(1) / R(12) - (iz * iz) * (R(1) / R(360)));
+      return lhs <= rhs;
+    }
   }
-  return lhs <= rhs;
+  const R loglam = P::log(mu);
+  return lhs <= (-mu + kd * loglam) - P::lfact(count_of(kd));
 }
 
 // The same test estimated in FP32: 1 accept, -1 reject, 0 too close to tell (then the caller
@@ -581,17 +581,12 @@ __device__ __forceinline__ long long poisson_draw(typename P::R mu, uint32_t k0,
   return d.k;
 }
 
-// |a| > |b| (false when a is NaN)
-__device__ __forceinline__ bool abs_gt(double a, double b) { return f64_abs_gt(a, b); }
-__device__ __forceinline__ bool abs_gt(float a, float b) { return fabsf(a) > fabsf(b); }
-
 // v t for a net change v: the common changes by one are exact without a product.
 __device__ __noinline__ inline double nu_times_call(int v, double t) { return f64_of_i32(v) * t; }
 __device__ __forceinline__ double nu_times(int v, double t) {
   return v == 1 ? t : v == -1 ? -t : v == 2 ? 2.0 * t : v == -2 ? -2.0 * t
                                                                 : nu_times_call(v, t);
 }
-__device__ __forceinline__ float nu_times(int v, float t) { return (float)v * t; }
 
 // MDL: the model tables' type -- the shared-memory ThreadModel staged at kernel start, or
 // a type with the same members known at compile time.
@@ -889,7 +884,7 @@ struct ThreadTraj {
         R best = fabs(A[k][k]);
 #pragma unroll
         for (int i = k + 1; i < NM; ++i) {
-          if (abs_gt(A[i][k], best)) {
+          if (f64_abs_gt(A[i][k], best)) {
             best = fabs(A[i][k]);
             piv = i;
           }

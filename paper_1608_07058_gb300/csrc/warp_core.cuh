@@ -797,8 +797,7 @@ struct WarpTraj {
     // The propensities come from an FP32 copy of the state (kept in the leap's xn storage,
     // unused during a burst, and updated with each firing), one FP32 warp scan gives a0
     // and the pick, and the next firing's random block is generated one firing ahead.
-    auto ssa_burst_fast = [&](int n_max, R a0_unused) {
-      (void)a0_unused;
+    auto ssa_burst_fast = [&](int n_max) {
       const double rem = T - t;
       const float remf = f32_of_f64(rem);
       float el = 0.f, elc = 0.f;
@@ -891,7 +890,7 @@ struct WarpTraj {
 
     auto ssa_burst = [&](int n_max, R a0) {
       if (!P::kRef) {
-        ssa_burst_fast(n_max, a0);
+        ssa_burst_fast(n_max);
         return;
       }
       int fired = -1;
