@@ -181,9 +181,9 @@ NEWTON_ITERATIONS = 4.3  # mean iterations per implicit leap on dimerisation sta
 # reports null.  Captures: the full 1,000,000-trajectory batch, one launch each, CTAs per
 # SM by occupancy.
 _SRC = ("ncu --metrics gpu__time_duration.sum,smsp__inst_executed.sum,dram__bytes_read.sum,"
-        "dram__bytes_write.sum,sm__inst_executed_pipe_fp64... -k regex:ml_jit -s 1 -c 1 "
-        "python bench.py --config 2 --steps 1 --warmup 1 --no-plain --no-cpu "
-        "--serving-seconds 0 --ncu --shape S --block B "
+        "dram__bytes_write.sum,sm__inst_executed_pipe_fp64... --clock-control none "
+        "-k regex:ml_jit -s 1 -c 1 python bench.py --config 2 --steps 1 --warmup 1 "
+        "--no-plain --no-cpu --serving-seconds 0 --ncu --shape S --block B "
         "(profiles/k_jit_pool_fast_gene_expression_1M.md)")
 PROFILED = {
     (2, 6, 64, 1): {"dram_bytes": 280674048 + 247611136, "warp_inst": 100004762963,

@@ -478,8 +478,8 @@ __device__ __noinline__ PoissonDraw poisson_ptrs(typename P::R mu, uint32_t k0, 
 // distance of mu / k from a midpoint of two numbers: mu / k = c/k ulps with an integer c, so
 // it is no midpoint (k times an odd half-integer of the quotient's precision does not fit
 // the significand of mu) and at least 1/(2k) ulp away from one.  So the result is that
-// of the IEEE division, in 4 instructions instead of about 10 (FP32) and in 3 on the
-// FP64 unit instead of 9 and a conversion of k.
+// of the IEEE division, in 4 instructions (FP32), or in 3 on the FP64 unit (192 of its
+// cycles; a division occupies it for 564) and a conversion of k on the integer pipe.
 __device__ __forceinline__ float div_by_int(float mu, int k) {
   const float kf = (float)k;
   const float z = __fdividef(1.f, kf);
