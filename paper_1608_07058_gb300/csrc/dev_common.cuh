@@ -113,13 +113,12 @@ __device__ __forceinline__ double f64_of_i32(int k) {
   return __hiloint2double((int)(a ? h : 0u), (int)(m << 21));
 }
 
-// t < T for a time t in [0, +inf] or NaN and a horizon T that is not NaN (it may be negative):
-// as unsigned integers with the sign shifted out.  0 inf gives a NaN whose sign is set, which
-// as a signed integer lies below every T; the absolute value may be an FP64 instruction and
-// leave that sign.
+// t < T for a time t in [0, +inf] (not -0) or NaN and a horizon T that is not NaN (it may be
+// negative): as integers, false for a NaN of either sign (0 inf gives one whose sign is set,
+// which lies below every number; the other lies above).
 __device__ __forceinline__ bool before_horizon(double t, double T) {
-  const long long bT = __double_as_longlong(T);
-  return bT > 0 && ((unsigned long long)__double_as_longlong(t) << 1) < ((unsigned long long)bT << 1);
+  const long long bt = __double_as_longlong(t);
+  return bt >= 0 && bt < __double_as_longlong(T);
 }
 
 // tn > T for a time tn in [0, +inf] (not -0) or NaN of either sign and a horizon T > 0: false

@@ -74,12 +74,16 @@ __device__ inline WarpSlab carve_slab(char* p, int N, int M, int rbytes, int lby
   return s;
 }
 
-// Comparisons of the Newton system on the integer pipe: a > b where each is not negative or
-// -1 (no row) and b is not NaN, false when a is NaN of either sign; equality of values that
-// are not NaN; zero.
+// Comparisons of the Newton system on the integer pipe.  |a| as a pivot's size: -1 (no row)
+// for a NaN of either sign, so that sizes are not negative or -1; a > b of two sizes; equality
+// of two; zero.
+__device__ __forceinline__ double pivot_size(double a) {
+  const double v = fabs(a);
+  return ((unsigned long long)__double_as_longlong(v) << 1) <= 0xffe0000000000000ULL ? v : -1.0;
+}
+__device__ __forceinline__ float pivot_size(float a) { return fabsf(a); }
 __device__ __forceinline__ bool pivot_gt(double a, double b) {
-  const long long ua = __double_as_longlong(a);
-  return ua > __double_as_longlong(b) && ((unsigned long long)ua << 1) <= 0xffe0000000000000ULL;
+  return __double_as_longlong(a) > __double_as_longlong(b);
 }
 __device__ __forceinline__ bool pivot_gt(float a, float b) { return a > b; }
 __device__ __forceinline__ bool same_bits(double a, double b) {
@@ -500,7 +504,7 @@ struct WarpTraj {
         for (int q = 0; q < kSPL; ++q) {
           const int i = k + lane + 32 * q;
           own_v[q] = i < N ? Jm[(size_t)i * N + k] : L(0);
-          const L v = fabs(own_v[q]);
+          const L v = pivot_size(own_v[q]);
           if (i < N && pivot_gt(v, best)) {
             best = v;
             piv = i;
