@@ -186,12 +186,14 @@ _SRC = ("ncu --metrics gpu__time_duration.sum,smsp__inst_executed.sum,dram__byte
         "--no-plain --no-cpu --serving-seconds 0 --ncu --shape S --block B "
         "(profiles/k_jit_pool_fast_gene_expression_1M.md)")
 PROFILED = {
-    (2, 6, 64, 1): {"dram_bytes": 280674048 + 247611136, "warp_inst": 100004762963,
-                    "fp64_pipe_pct": 12.21, "source": _SRC},
-    (2, 6, 128, 1): {"dram_bytes": 280562432 + 248731648, "warp_inst": 100010507863,
+    (2, 6, 64, 1): {"dram_bytes": 279840000 + 247480000, "warp_inst": 100055639727,
+                    "fp64_pipe_pct": 12.19, "source": _SRC},
+    (2, 6, 128, 1): {"dram_bytes": 283100000 + 248760000, "warp_inst": 100153525883,
                      "fp64_pipe_pct": 12.20, "source": _SRC},
-    (2, 7, 64, 1): {"dram_bytes": 300612864 + 2831970048, "warp_inst": 108139420645,
-                    "fp64_pipe_pct": 14.24, "source": _SRC},
+    (2, 6, 256, 1): {"dram_bytes": 278320000 + 247370000, "warp_inst": 100124456322,
+                     "fp64_pipe_pct": 12.19, "source": _SRC},
+    (2, 7, 64, 1): {"dram_bytes": 301520000 + 2850000000, "warp_inst": 108157438181,
+                    "fp64_pipe_pct": 14.10, "source": _SRC},
 }
 
 
