@@ -128,7 +128,8 @@ __device__ __forceinline__ bool past_horizon(double tn, double T) {
   return bt > __double_as_longlong(T) && bt <= 0x7ff0000000000000LL;
 }
 
-// a < b for operands that are each in [0, +inf] (not -0) or NaN.
+// a < b for operands that are each in [0, +inf] (not -0) or NaN of either sign.  Unsigned: the
+// mask may be compiled to an FP64 absolute value, which leaves a NaN's sign.
 __device__ __forceinline__ bool f64_lt_pos(double a, double b) {
   const unsigned long long m = 0x7fffffffffffffffULL, inf = 0x7ff0000000000000ULL;
   const unsigned long long ub = (unsigned long long)__double_as_longlong(b) & m;

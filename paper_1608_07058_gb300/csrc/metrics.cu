@@ -76,13 +76,13 @@ __device__ __forceinline__ void for_samples(const int64_t* __restrict__ x, long 
   for (; i < n; i += kKlThreads) f(x[i * stride]);
 }
 
-// One CTA per (time point k, species s).  X layout [n][K][N].  10,000 trajectories of 20
-// points and 3 species (60 CTAs, 9.6 MB) took 124 us with 256 threads, one load in flight
-// each and one warp taking two FP64 logarithms and two divisions per bin: about 120
-// instructions of 64 cycles on the FP64 unit for each 32 of some 700 bins.  Now the
-// probabilities and logarithms are computed once per distinct count (a bin holds at most a
-// few dozen of the samples, and the tails' bins hold the same few counts) by all warps, and
-// the terms by all warps; one warp only adds them in the canonical order.
+// One CTA per (time point k, species s).  X layout [n][K][N].  The probabilities and
+// logarithms are computed once per distinct count (a bin holds at most a few dozen of the
+// samples, and the tails' bins hold the same few counts) by all warps, and the terms by all
+// warps; one warp only adds them in the canonical order.  10,000 trajectories of 20 points and
+// 3 species (60 CTAs, 9.6 MB): 40 us, bound by the latency of the strided loads; 124 us with
+// 256 threads, one load in flight each and one warp taking two logarithms and two divisions
+// per bin (about 120 instructions of 64 cycles on the FP64 unit for each 32 of some 700 bins).
 __global__ void __launch_bounds__(kKlThreads) k_kl(int64_t n_ref, const int64_t* __restrict__ Xr,
                                                   int64_t n_test, const int64_t* __restrict__ Xt,
                                                   int K, int N, int max_bins,

@@ -596,9 +596,9 @@ struct ThreadTraj {
   using Model = MDL;
 
   // g_j of a state by the table's reactant word: comb(x_s, m) of the k-th reactant, the
-  // product in increasing s, 0 when some x_s < m_js.  The code is a tenth of the loop over
-  // all (reaction, species) pairs with a branch per order, which the precompiled kernels
-  // ran before: their stalls were instruction fetch.
+  // product in increasing s, 0 when some x_s < m_js.  The code is a tenth of a loop over
+  // all (reaction, species) pairs with a branch per order, on which the precompiled kernels
+  // stall in instruction fetch.
   // Orders above two are out of line (bit 31 of the word).
   template <class V>
   __device__ static __forceinline__ V sel(const V (&x)[NM], int sp) {
