@@ -506,9 +506,12 @@ struct Plan {
 //                 8 x 16 kernel   4 units 0.69 (0.52-1.03), 6.6 1.04 (0.81-1.55)
 //     plain (no refill of a warp)
 //                 <= 4 reactions  3 units 0.92 (0.74-1.32), 4 1.07
-//                 more            4 units 0.84 (0.50-1.36), 6.6 1.11 (0.57-2.02)
+//                 5, 6 reactions  6 units 0.99 (0.59-1.70), 6.6 0.97 (0.57-2.02), 7.4 1.12
+//                 8 x 16 kernel   4 units 0.76 (0.50-1.18), 6.6 1.16
 //     thread kernel compiled for the model
-//                                 2 units 0.81 (0.57-1.14), 3 0.99 (0.79-1.22);
+//                 <= 4 reactions  2 units 0.83 (0.74-0.89), 4 1.06
+//                 5, 6 reactions  3 units 0.86 (0.68-1.24), 4 0.94 (0.64-1.53)
+//                 8 x 16 kernel   2 units 0.84 (0.57-1.14), 3 1.05;
 //   own rate constants and one horizon, or the reverse
 //                           1 unit 0.51 (0.18-0.81), 2 units 0.69 (0.29-1.25): 1 too.
 // Gene expression, 10,007 own rate constants and horizons: 530 ms on threads, 352 on warps;
@@ -530,10 +533,12 @@ int64_t ref_warp_limit(const ml_model& m, DeviceState& st, const ml_sim_params& 
   if (persistent && p.ctas_per_sm)
     per_sm = std::min(per_sm, p.ctas_per_sm * (p.block_size ? p.block_size : 128) / 32);
   if (!ragged) return (int64_t)st.sm_count * per_sm;
-  // rows: kernels for up to 4 reactions, for 5 and 6 (3 species), 8 x 16
-  static constexpr int kUnits[3][2] = {{3, 4}, {5, 9}, {5, 6}};  // plain, persistent
-  const int row = mlk::kThreadM[m.thread_variant] <= 4 ? 0 : mlk::kThreadM[m.thread_variant] <= 6 ? 1 : 2;
-  const int units = p.specialize && !grid_out ? 2 : kUnits[row][persistent ? 1 : 0];
+  // rows: kernels for up to 4 reactions, for 5 and 6 (3 species), 8 x 16; columns: thread
+  // kernel compiled for the model, plain, persistent
+  static constexpr int kUnits[3][3] = {{2, 3, 4}, {4, 7, 9}, {2, 5, 6}};
+  const int M = mlk::kThreadM[m.thread_variant];
+  const int units = kUnits[M <= 4 ? 0 : M <= 6 ? 1 : 2]
+                          [p.specialize && !grid_out ? 0 : persistent ? 2 : 1];
   return (int64_t)st.sm_count * per_sm * units;
 }
 
